@@ -188,7 +188,7 @@ struct GemmArgs {
   const char* name;                  // label for per-launch profiling (nullptr = by epilogue)
 };
 cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s);    // bf16, tcgen05
-cudaError_t launch_gemm_simt(const GemmArgs& a, int epi, cudaStream_t s);  // fp32, CUDA cores
+cudaError_t launch_gemm_f32(const GemmArgs& a, int epi, cudaStream_t s);   // fp32 through three bf16 terms, tcgen05
 // bf16 groups of at most 16 rows (decode batches): weight rows streamed once
 // on the CUDA cores; every epilogue but EPI_REPLICATE.
 bool gemm_skinny_supported(const GemmArgs& a, int epi);
@@ -241,12 +241,12 @@ cudaError_t read_codec_error(unsigned int* word);
 cudaError_t read_gate_error(unsigned int* word);
 
 // Reads and clears the tensor-core kernels' device error word (synchronous).
-// In the grouped-GEMM words (tensor-core, swapped, weight-streaming, SIMT)
+// In the grouped-GEMM words (tensor-core, swapped, weight-streaming, fp32)
 // bit 0 is a timed-out wait and bit 1 a group range (offsets) or a scatter
 // destination (perm) outside the call's rows, skipped.
 cudaError_t read_tc_error(unsigned int* word);
 cudaError_t read_skinny_error(unsigned int* word);
-cudaError_t read_simt_error(unsigned int* word);
+cudaError_t read_f32_error(unsigned int* word);
 // Reads and clears the routing kernels' device error word (synchronous):
 // nonzero when an expert id outside [0, E) or a permutation entry outside
 // [0, rows) was met (and skipped).
