@@ -148,20 +148,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    // (producer and MMA warp: the whole warp waits and counts, so that addresses
+    // and descriptors stay in uniform registers; one elected lane issues)
+    {
+      const bool issue = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_phase = 0;
       bool ok = true;
       const int n_loads = K1 + K2;
       for (int i = 0; i < n_loads && ok; ++i) {
-        if (!mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_codec_error)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_codec_error))) {
           ok = false;
           break;
         }
         const uint32_t fb = smem_u32(&full[stage]);
         uint8_t* st = stages + stage * C::STAGE_BYTES;
-        if (i < K1) {
+        if (!issue) {
+        } else if (i < K1) {
           mbar_expect_tx(fb, C::A_BYTES + R * BK * 2);
           tma_load_2d(smem_u32(st), &tmX, i * BK, m0, fb);
           tma_load_2d(smem_u32(st + C::A_BYTES), &tmVe, i * BK, 0, fb);
@@ -183,7 +188,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
+      const bool issue = elect_one();
       constexpr uint32_t IDESC_Z = idesc_bf16(BM, R);
       constexpr uint32_t IDESC_X = idesc_bf16(BM, BN);
       int stage = 0;
@@ -191,7 +197,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool ok = true, any = false;
       // Z = X V_enc^T
       for (int kb = 0; kb < K1 && ok; ++kb) {
-        if (!mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_codec_error)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_codec_error))) {
           ok = false;
           break;
         }
@@ -199,24 +206,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const uint8_t* st = stages + stage * C::STAGE_BYTES;
         const uint64_t da = sdesc_sw128(smem_u32(st));
         const uint64_t db = sdesc_sw128(smem_u32(st + C::A_BYTES));
+        if (issue) {
 #pragma unroll
-        for (int kk = 0; kk < BK / UK; ++kk)
-          umma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC_Z, (kb | kk) != 0 ? 1u : 0u);
+          for (int kk = 0; kk < BK / UK; ++kk)
+            umma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC_Z, (kb | kk) != 0 ? 1u : 0u);
+          umma_commit(smem_u32(&empty[stage]));
+        }
         any = true;
-        umma_commit(smem_u32(&empty[stage]));
         if (++stage == C::STAGES) {
           stage = 0;
           phase ^= 1u;
         }
       }
       if (ok) {
-        umma_commit(smem_u32(zfull));
+        if (issue) umma_commit(smem_u32(zfull));
         // X_hat = Z V_dec^T once the epilogue has put Z (bf16) in shared memory
-        ok = mbar_wait(smem_u32(zready), 0, budget, abort_flag, &g_codec_error);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(zready), 0, budget, abort_flag, &g_codec_error));
         tc_fence_after();
       }
       for (int kb = 0; kb < K2 && ok; ++kb) {
-        if (!mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_codec_error)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_codec_error))) {
           ok = false;
           break;
         }
@@ -224,17 +234,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const uint8_t* st = stages + stage * C::STAGE_BYTES;
         const uint64_t da = sdesc_sw128(smem_u32(zs + kb * (BM * 128)));
         const uint64_t db = sdesc_sw128(smem_u32(st + C::A_BYTES));
+        if (issue) {
 #pragma unroll
-        for (int kk = 0; kk < BK / UK; ++kk)
-          umma_bf16(tmem_base + X_ACC_COL, da + 2 * kk, db + 2 * kk, IDESC_X, (kb | kk) != 0 ? 1u : 0u);
-        umma_commit(smem_u32(&empty[stage]));
+          for (int kk = 0; kk < BK / UK; ++kk)
+            umma_bf16(tmem_base + X_ACC_COL, da + 2 * kk, db + 2 * kk, IDESC_X, (kb | kk) != 0 ? 1u : 0u);
+          umma_commit(smem_u32(&empty[stage]));
+        }
         if (++stage == C::STAGES) {
           stage = 0;
           phase ^= 1u;
         }
       }
-      if (ok) umma_commit(smem_u32(xfull));
-      if ((!ok || *abort_flag) && any) {
+      if (ok && issue) umma_commit(smem_u32(xfull));
+      if ((!ok || *abort_flag) && any && issue) {
         umma_commit(smem_u32(drain));
         mbar_drain(smem_u32(drain), 0, DRAIN_CYCLES);
       }

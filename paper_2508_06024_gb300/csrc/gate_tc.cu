@@ -584,7 +584,10 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // the whole warp waits and counts, so that descriptors stay in uniform
+    // registers; one elected lane issues
+    {
+      const bool issue = elect_one();
       const uint32_t idesc = idesc_bf16(GC_BM, 3 * n_pad);
       int stage = 0;
       uint32_t phase = 0;
@@ -594,7 +597,8 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
       for (int tile = tile_first; tile < n_tiles && ok; tile += tile_step) {
         for (int seg = 0; seg < cnt && ok; seg += GC_SEG) {
           const uint32_t uses = acc ? uses1 : uses0;
-          if (!mbar_wait(smem_u32(&tempty[acc]), (uses & 1u) ^ 1u, budget, abort_flag, &g_gate_error)) {
+          if (!__all_sync(0xffffffffu,
+                          mbar_wait(smem_u32(&tempty[acc]), (uses & 1u) ^ 1u, budget, abort_flag, &g_gate_error))) {
             ok = false;
             break;
           }
@@ -602,8 +606,10 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
           const uint32_t d_tmem = tmem_base + acc * GC_ACC_STRIDE;
           const int seg_end = seg + GC_SEG < cnt ? seg + GC_SEG : cnt;
           for (int kc = seg; kc < seg_end; ++kc) {
-            if ((!PREP && !mbar_wait(smem_u32(&conv[stage]), phase, budget, abort_flag, &g_gate_error)) ||
-                !mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_gate_error)) {
+            const bool landed =
+                (PREP || mbar_wait(smem_u32(&conv[stage]), phase, budget, abort_flag, &g_gate_error)) &&
+                mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_gate_error);
+            if (!__all_sync(0xffffffffu, landed)) {
               ok = false;
               break;
             }
@@ -611,24 +617,26 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
             const uint8_t* st = smem + stage * L.stage_bytes;
             const uint64_t da = sdesc_sw128(smem_u32(st));
             const uint64_t db = sdesc_sw128(smem_u32(st + L.w3_off));
+            if (issue) {
 #pragma unroll
-            for (int kk = 0; kk < GC_BK / 16; ++kk)
-              umma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (kc != seg || kk != 0) ? 1u : 0u);
+              for (int kk = 0; kk < GC_BK / 16; ++kk)
+                umma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (kc != seg || kk != 0) ? 1u : 0u);
+              umma_commit(smem_u32(&empty[stage]));
+            }
             any = true;
-            umma_commit(smem_u32(&empty[stage]));
             if (++stage == S) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          umma_commit(smem_u32(&tfull[acc]));
+          if (issue) umma_commit(smem_u32(&tfull[acc]));
           if (acc) ++uses1;
           else ++uses0;
           acc ^= 1;
         }
       }
-      if ((!ok || *abort_flag) && any) {
+      if ((!ok || *abort_flag) && any && issue) {
         umma_commit(smem_u32(drain));
         mbar_drain(smem_u32(drain), 0, DRAIN_CYCLES);
       }

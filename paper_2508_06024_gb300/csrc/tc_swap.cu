@@ -195,7 +195,9 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    // The whole warp waits and counts; one elected lane issues.
+    {
+      const bool issue = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0;  // bit s: stage s holds a copy the consumer has not released
@@ -209,21 +211,20 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
         const int kb0 = un.ks * p.kb_per_split;
         const int kb1 = kb0 + p.kb_per_split < num_kb ? kb0 + p.kb_per_split : num_kb;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_swap_error)) {
+          if (!__all_sync(0xffffffffu,
+                          mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_swap_error))) {
             ok = false;
             break;
           }
           const uint32_t fb = smem_u32(&full[stage]);
-          mbar_expect_tx(fb, SW_STAGE_BYTES);
           const uint32_t dw = smem_u32(sW + stage * SW_W_BYTES);
-          if (GLU) {
+          if (issue) {
+            mbar_expect_tx(fb, SW_STAGE_BYTES);
+            tma_load_2d(dw, &tmW, kb * SW_BK, w_row, fb);
             // rows 0-63 of the tile: W1, rows 64-127: W3, same output columns
-            tma_load_2d(dw, &tmW, kb * SW_BK, w_row, fb);
-            tma_load_2d(dw + SW_W_BYTES / 2, &tmW2, kb * SW_BK, w_row, fb);
-          } else {
-            tma_load_2d(dw, &tmW, kb * SW_BK, w_row, fb);
+            if (GLU) tma_load_2d(dw + SW_W_BYTES / 2, &tmW2, kb * SW_BK, w_row, fb);
+            tma_load_2d(smem_u32(sX + stage * SW_X_BYTES), &tmX, kb * SW_BK, x_row, fb);
           }
-          tma_load_2d(smem_u32(sX + stage * SW_X_BYTES), &tmX, kb * SW_BK, x_row, fb);
           issued |= 1u << stage;
           issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == SW_STAGES) {
@@ -239,8 +240,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       // ---------------------------------------------------------------- MMA issuer
+      // The whole warp waits and counts, so that descriptors stay in uniform
+      // registers; one elected lane issues.
+      const bool issue = elect_one();
       constexpr uint32_t IDESC = idesc_bf16(SW_M, SW_N);
       const uint64_t dw0 = sdesc_sw128(smem_u32(sW));
       const uint64_t dx0 = sdesc_sw128(smem_u32(sX));
@@ -254,14 +258,15 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
         const int kb1 = kb0 + p.kb_per_split < num_kb ? kb0 + p.kb_per_split : num_kb;
         const int acc = it % SW_ACC;
         const uint32_t acc_phase = static_cast<uint32_t>(it / SW_ACC) & 1u;
-        if (!mbar_wait(smem_u32(&tempty[acc]), acc_phase ^ 1u, budget, abort_flag, &g_swap_error)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&tempty[acc]), acc_phase ^ 1u, budget, abort_flag, &g_swap_error))) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * SW_N);
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_swap_error)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_swap_error))) {
             ok = false;
             break;
           }
@@ -271,20 +276,22 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
           // addresses are below 256 KB)
           const uint64_t da = dw0 + static_cast<uint64_t>(stage) * (SW_W_BYTES >> 4);
           const uint64_t db = dx0 + static_cast<uint64_t>(stage) * (SW_X_BYTES >> 4);
-          umma_bf16(d_tmem, da, db, IDESC, kb != kb0 ? 1u : 0u);
+          if (issue) {
+            umma_bf16(d_tmem, da, db, IDESC, kb != kb0 ? 1u : 0u);
 #pragma unroll
-          for (int kk = 1; kk < SW_BK / SW_UK; ++kk) umma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, IDESC, 1u);
+            for (int kk = 1; kk < SW_BK / SW_UK; ++kk) umma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, IDESC, 1u);
+            umma_commit(smem_u32(&empty[stage]));
+          }
           any = true;
-          umma_commit(smem_u32(&empty[stage]));
           if (++stage == SW_STAGES) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&tfull[acc]));
+        if (issue) umma_commit(smem_u32(&tfull[acc]));
       }
-      if ((!ok || *abort_flag) && any) {
+      if ((!ok || *abort_flag) && any && issue) {
         // All MMAs issued so far must finish before TMEM is freed.
         umma_commit(smem_u32(drain));
         mbar_drain(smem_u32(drain), 0, DRAIN_CYCLES);
