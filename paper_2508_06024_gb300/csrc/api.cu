@@ -353,6 +353,7 @@ cudaError_t run_gemm(const ec2moe_layer_desc* d, const GemmArgs& g, int epi, cud
   // streamed once on the CUDA cores
   if (gemm_swap_supported(g, epi)) return launch_gemm_swap(g, epi, s);
   if (gemm_skinny_supported(g, epi)) return launch_gemm_skinny(g, epi, s);
+  if (tok_gemm_preferred(g, epi)) return launch_gemm_tok(g, epi, s);
   return launch_gemm_tc(g, epi, s);
 }
 
@@ -1026,7 +1027,7 @@ ec2moe_status ec2moe_layer_forward_pipelined(const ec2moe_layer_desc* desc, cons
 
 ec2moe_status ec2moe_last_device_error(ec2moe_stream_t stream) {
   if (cudaStreamSynchronize(stream) != cudaSuccess) return EC2MOE_ERR_CUDA;
-  unsigned int tc = 0, codec = 0, gate = 0, route = 0, swap = 0, skinny = 0, f32 = 0;
+  unsigned int tc = 0, codec = 0, gate = 0, route = 0, swap = 0, skinny = 0, f32 = 0, tok = 0;
   if (read_tc_error(&tc) != cudaSuccess) return EC2MOE_ERR_CUDA;
   if (read_codec_error(&codec) != cudaSuccess) return EC2MOE_ERR_CUDA;
   if (read_gate_error(&gate) != cudaSuccess) return EC2MOE_ERR_CUDA;
@@ -1034,11 +1035,12 @@ ec2moe_status ec2moe_last_device_error(ec2moe_stream_t stream) {
   if (read_swap_error(&swap) != cudaSuccess) return EC2MOE_ERR_CUDA;
   if (read_skinny_error(&skinny) != cudaSuccess) return EC2MOE_ERR_CUDA;
   if (read_f32_error(&f32) != cudaSuccess) return EC2MOE_ERR_CUDA;
+  if (read_tok_error(&tok) != cudaSuccess) return EC2MOE_ERR_CUDA;
   // bit 0 of the GEMM, codec and gate words: a bounded wait timed out;
   // bit 1 of the GEMM words and any bit of the routing word: an index outside
   // the call's rows or experts was skipped
-  if ((tc | codec | gate | swap | f32) & 1u) return EC2MOE_ERR_TIMEOUT;
-  if (((tc | swap | skinny | f32) & 2u) || route) return EC2MOE_ERR_INVALID_ARG;
+  if ((tc | codec | gate | swap | f32 | tok) & 1u) return EC2MOE_ERR_TIMEOUT;
+  if (((tc | swap | skinny | f32 | tok) & 2u) || route) return EC2MOE_ERR_INVALID_ARG;
   return EC2MOE_OK;
 }
 

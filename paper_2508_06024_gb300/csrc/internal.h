@@ -57,6 +57,31 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Clusters of `cdim` CTAs of `kernel` that fit on the device at once (cached
+// per device and kernel); 0 when the query fails.
+int max_clusters(const void* kernel, int threads, int smem, int cdim);
+
+// As launch_kernel, for `clusters` clusters of `cdim` CTAs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int clusters, int cdim, int threads, size_t smem,
+                                  cudaStream_t s, Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cdim * clusters);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cdim;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = next_launch_pdl() ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per (device, kernel),
 // raised only when a launch needs more than was set before.
 cudaError_t ensure_smem_attr(const void* kernel, int bytes);
@@ -189,6 +214,13 @@ struct GemmArgs {
 };
 cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s);    // bf16, tcgen05
 cudaError_t launch_gemm_f32(const GemmArgs& a, int epi, cudaStream_t s);   // fp32 through three bf16 terms, tcgen05
+// bf16 with the weights on the MMA's M side and a group's tokens on its N side
+// (CTA pairs); EPI_STORE, GELU, SWIGLU and SCATTER.  tok_gemm_preferred:
+// whether it is the better one for this call (else launch_gemm_tc).
+bool gemm_tok_supported(const GemmArgs& a, int epi);
+bool tok_gemm_preferred(const GemmArgs& a, int epi);
+cudaError_t launch_gemm_tok(const GemmArgs& a, int epi, cudaStream_t s);
+cudaError_t read_tok_error(unsigned int* word);
 // bf16 groups of at most 16 rows (decode batches): weight rows streamed once
 // on the CUDA cores; every epilogue but EPI_REPLICATE.
 bool gemm_skinny_supported(const GemmArgs& a, int epi);

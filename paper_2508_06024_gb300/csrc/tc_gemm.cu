@@ -795,62 +795,6 @@ const char* kernel_name(int epi) {
   }
 }
 
-// Clusters of `cdim` CTAs (2: one pair, 4: two pairs) of `kernel` that fit on
-// the device at once (cached per device and kernel); 0 when the query fails.
-int max_pair_clusters(const void* kernel, int smem, int cdim) {
-  struct Entry {
-    int dev;
-    const void* kernel;
-    int n;
-  };
-  static std::mutex mu;
-  static Entry cache[32];
-  static int used = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> lock(mu);
-  for (int i = 0; i < used; ++i)
-    if (cache[i].dev == dev && cache[i].kernel == kernel) return cache[i].n;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(cdim * sm_count());
-  cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cdim;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    n = 0;
-  }
-  if (used < 32) cache[used++] = Entry{dev, kernel, n};
-  return n;
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pairs(void (*kernel)(KArgs...), int clusters, int cdim, size_t smem, cudaStream_t s,
-                         Args&&... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(cdim * clusters);
-  cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cdim;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = next_launch_pdl() ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 template <int BN, int EPI, int STAGES, bool PAIR = false, bool QUAD = false>
 cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   using C = Cfg<BN, EPI, STAGES, PAIR>;
@@ -904,12 +848,12 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
     // QUAD: a cluster tile is two N tiles (p.n_tiles_n is even)
     if (QUAD) tiles /= 2;
     const int cdim = QUAD ? 4 : 2;
-    int clusters = max_pair_clusters(kfn, C::SMEM, cdim);
+    int clusters = max_clusters(kfn, NUM_THREADS, C::SMEM, cdim);
     if (clusters < 1) return cudaErrorInvalidConfiguration;
     if (tiles < clusters) clusters = static_cast<int>(tiles < 1 ? 1 : tiles);
     KernelScope ks(a.name ? a.name : kernel_name(EPI), s);
-    cudaError_t le = launch_pairs(tc_gemm_kernel<BN, EPI, STAGES, PAIR, QUAD>, clusters, cdim, (size_t)C::SMEM, s, mA,
-                                  mB, mB2, p);
+    cudaError_t le = launch_cluster(tc_gemm_kernel<BN, EPI, STAGES, PAIR, QUAD>, clusters, cdim, NUM_THREADS,
+                                    (size_t)C::SMEM, s, mA, mB, mB2, p);
     if (le != cudaSuccess) return le;
     return cudaGetLastError();
   }
@@ -985,6 +929,42 @@ int choose_bn(const GemmArgs& a, int epi, bool pair = false) {
 }
 
 }  // namespace
+
+// Clusters of `cdim` CTAs (2: one pair, 4: two pairs) of `kernel` that fit on
+// the device at once (cached per device and kernel); 0 when the query fails.
+int max_clusters(const void* kernel, int threads, int smem, int cdim) {
+  struct Entry {
+    int dev;
+    const void* kernel;
+    int n;
+  };
+  static std::mutex mu;
+  static Entry cache[32];
+  static int used = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < used; ++i)
+    if (cache[i].dev == dev && cache[i].kernel == kernel) return cache[i].n;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cdim * sm_count());
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cdim;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    n = 0;
+  }
+  if (used < 32) cache[used++] = Entry{dev, kernel, n};
+  return n;
+}
 
 bool make_tensor_map_bf16(CUtensorMap* m, const void* ptr, long long rows, long long cols, int box_rows) {
   return make_map(m, ptr, rows, cols, box_rows, MAP_BF16_SW128);
