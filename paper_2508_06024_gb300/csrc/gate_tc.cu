@@ -37,8 +37,8 @@ namespace {
 //   warp 0       TMA: the X box (128 x 64 bf16, 128-byte swizzle) and the
 //                stacked split rows of the stage -- either straight from a
 //                prepared [3 * O_pad, d] bf16 matrix (PREP: made by
-//                gate_split_kernel), or as raw fp32 rows (O x 64, unswizzled)
-//                that warps 6..13 split into the swizzled layout;
+//                gate_split_kernel); without one, warps 6..13 load the fp32
+//                rows and write their split into the swizzled layout;
 //   warp 1       4 MMAs (M = 128, N = 3 O_pad, K = 16) per stage into one of
 //                two TMEM accumulators; every GC_SEG stages (256 columns of
 //                d_model) the accumulator is handed over and the next segment
@@ -46,9 +46,9 @@ namespace {
 //   warps 2..5   add each segment into fp32 registers (one token row per
 //                thread; warp w reads TMEM lanes 32 (w % 4) .. +31), so every
 //                dot product is a sum of short partial sums; at the end of the
-//                tile add the bias and take the token's softmax / Top-k
-//                decision (decide_token_thread);
-//   warps 2..13  on the layer path, reserve the tile's rows per expert.
+//                tile they add the bias and write the logits rows;
+//   warps 2..13  take the softmax / Top-k decisions (lse_rows, pick_row) and, on
+//                the layer path, reserve the tile's rows per expert.
 // With d_model of 2048 or more (32 or more stages per tile) a tile belongs to
 // a cluster of GC_CS CTAs on as many SMs instead: CTA c of the cluster runs
 // the stages [c nk / GC_CS, (c + 1) nk / GC_CS) and owns the decisions of
@@ -76,16 +76,15 @@ constexpr int GC_SPLIT_MIN_NK = 32; // stages per tile from which d_model is spl
 
 struct GcLayout {
   int n_pad, O, k, E, stages, cs;
-  int stage_bytes, w3_off, raw_off;
+  int stage_bytes, w3_off;
   int log_stride;  // logits row of a token: O logits + 16 group scratch words, odd (conflict-free rows)
   int rstride;     // floats per received partial-logit row: n_pad + 4 (16-byte rows, shifted banks)
-  int log_off, idx_off, tab_off, base_off, bias_off, recv_off, bar_off, total;
-  __host__ __device__ GcLayout(int O_, int k_, int E_, int stages_, bool prep, int cs_)
+  int log_off, idx_off, tab_off, base_off, bias_off, list_off, recv_off, bar_off, warm_off, total;
+  __host__ __device__ GcLayout(int O_, int k_, int E_, int stages_, int cs_)
       : O(O_), k(k_), E(E_), stages(stages_), cs(cs_) {
     n_pad = (O + 15) / 16 * 16;
     w3_off = GC_BM * GC_BK * 2;
-    raw_off = w3_off + 3 * n_pad * 128;
-    stage_bytes = raw_off + (prep ? 0 : n_pad * 256);  // a multiple of 1024
+    stage_bytes = w3_off + 3 * n_pad * 128;  // a multiple of 1024
     log_stride = (O + 16) | 1;
     rstride = n_pad + 4;
     log_off = stages * stage_bytes;
@@ -94,9 +93,12 @@ struct GcLayout {
     base_off = tab_off + (GC_BM * k / 32) * E * 4;
     bias_off = base_off + 4 * E;
     // received partials: [source CTA][owned row][rstride] (cs > 1)
-    recv_off = (bias_off + 4 * O + 15) / 16 * 16;
+    list_off = bias_off + 4 * O;  // allowed experts, then the first list place of each group
+    recv_off = (list_off + 4 * (E + 17) + 15) / 16 * 16;
     bar_off = (recv_off + (cs > 1 ? GC_BM * rstride * 4 : 0) + 7) / 8 * 8;
-    total = bar_off + (3 * stages + 6) * 8 + 16;
+    // a logits row of its own for the warm-up of the decision's code
+    warm_off = bar_off + (3 * stages + 6) * 8 + 16;
+    total = warm_off + (O + 16) * 4;
   }
 };
 
@@ -108,16 +110,25 @@ struct GcParams {
   long long timeout;
 };
 
-// One token's decision by one thread, from its logits row L[0..E) (local),
-// L[E..E+K) (global) and a scratch row G[0..K) -- the arithmetic of
-// decide_token_warp with sequential sums: per-group log-sum-exp over the
-// allowed members (Eq. 5), top-group pruning when top_groups > 0 (only the
-// top_groups live groups by m stay), log-sum-exp of the global logits over the
-// live (kept) groups (Eq. 6), key = (m_g - lse_g) + l_i (K = 1: l_i), weight
-// exp((m_g - LSE_m) + (l_i - lse_g)) (Eq. 7); Top-k by insertion into a sorted list (larger key
-// first, ties to the lower index).  Slots left empty by non-finite keys take
-// the lowest allowed experts not chosen yet.  The mask words are in
-// registers, so the loads of one pass are independent of each other.
+// The decision, from a tile's logits rows in shared memory (L[0..E) local,
+// L[E..E+K) global, then 16 scratch words G) and the list of allowed experts
+// in ascending order, cut into groups by s_grp[0..K].  Two steps:
+//   lse_rows   G[g] = log-sum-exp of group g's allowed members (Eq. 5), one
+//              (row, group) per thread, all worker threads; K = 1: the whole
+//              list as one group
+//   pick_row   one thread per row: top-group pruning when top_groups > 0 (only
+//              the top_groups live groups by m stay), log-sum-exp of the global
+//              logits over the live (kept) groups (Eq. 6), key = (m_g - lse_g) +
+//              l_i (K = 1: l_i), Top-k by insertion into a sorted list (larger
+//              key first, ties to the lower index), weight exp((m_g - LSE_m) +
+//              (l_i - lse_g)) (Eq. 7).  Slots left empty by non-finite keys take
+//              the lowest allowed experts not chosen yet.
+// The steps run once per tile, with code that the previous kernels' streams
+// have evicted from L2, so their size counts as much as their arithmetic: they
+// are rolled loops behind one call each, and an idle warp calls both on a
+// scratch row during the main loop, which brings the code to the SM before it
+// is needed.  (Fully unrolled per-thread decisions took 25 us of the
+// fine-grained gate and ~20 us of a 64-expert Top-1 one.)
 struct MaskRegs {
   uint32_t w0, w1, w2, w3;
   __device__ __forceinline__ bool has(int e) const {
@@ -146,13 +157,32 @@ __device__ __forceinline__ void topk_insert(float* tk, float* tl, int* ti, float
   }
 }
 
-// KS >= k slots are kept (KS in {1, 2, 4, 8}).
+__device__ __noinline__ void lse_rows(float* sLog, int log_stride, int O, const int* s_list, const int* s_grp, int K,
+                                      int row_lo, int n_rows, int wt, int threads) {
+#pragma unroll 1
+  for (int i = wt; i < n_rows * K; i += threads) {
+    const int r = i / K, g = i - r * K;
+    float* L = sLog + (row_lo + r) * log_stride;
+    const int lo = s_grp[g], hi = s_grp[g + 1];
+    float mx = -CUDART_INF_F;
+#pragma unroll 4
+    for (int j = lo; j < hi; ++j) mx = fmaxf(mx, L[s_list[j]]);
+    float sum = 0.0f;
+#pragma unroll 4
+    for (int j = lo; j < hi; ++j) sum += expf(L[s_list[j]] - mx);
+    L[O + g] = mx > -CUDART_INF_F ? mx + logf(sum) : -CUDART_INF_F;
+  }
+}
+
+// KS >= k slots are kept (KS in {1, 2, 4, 8}); `real` false: nothing is written
+// outside the row's scratch words.
 template <int KS>
-__device__ void decide_token_thread(int E, int K, int k, int renorm, int top_groups, const MaskRegs m, const float* L,
-                                    float* G, int32_t* topk_idx, float* topk_w, int tok, int* s_idx) {
-  const bool grouped = K > 1;
-  const int ng = grouped ? K : 1;
-  const int gsize = E / ng;
+__device__ __noinline__ void pick_row(const KParams& p, float* L, int O, const int* s_list, const int* s_grp, int tok,
+                                      int* s_idx, bool real) {
+  const bool grouped = p.K > 1;
+  const int ng = p.K;
+  const int k = p.k;
+  float* G = L + O;
   float tk[KS], tl[KS];
   int ti[KS];
 #pragma unroll
@@ -162,98 +192,73 @@ __device__ void decide_token_thread(int E, int K, int k, int renorm, int top_gro
     ti[j] = -1;
   }
   float lse_m = 0.0f;
-  if (!grouped) {
-    // one group: the keys are the logits themselves, so Top-k rides on the max pass
-    float mx = -CUDART_INF_F;
-#pragma unroll 1
-    for (int e = 0; e < E; ++e) {
-      if (!m.has(e)) continue;
-      const float le = L[e];
-      mx = fmaxf(mx, le);
-      if (le > tk[KS - 1]) topk_insert<KS>(tk, tl, ti, le, e, le);
-    }
-    float sum = 0.0f;
-#pragma unroll 1
-    for (int e = 0; e < E; ++e)
-      if (m.has(e)) sum += expf(L[e] - mx);
-    G[0] = mx + logf(sum);
-#pragma unroll
-    for (int j = 0; j < KS; ++j) tl[j] -= G[0];
-  } else {
-    float mxm = -CUDART_INF_F;
-#pragma unroll 1
-    for (int g = 0; g < ng; ++g) {
-      const int lo = g * gsize, hi = lo + gsize;
-      float mx = -CUDART_INF_F;
-#pragma unroll 4
-      for (int e = lo; e < hi; ++e)
-        if (m.has(e)) mx = fmaxf(mx, L[e]);
-      float sum = 0.0f;
-#pragma unroll 4
-      for (int e = lo; e < hi; ++e)
-        if (m.has(e)) sum += expf(L[e] - mx);
-      G[g] = mx > -CUDART_INF_F ? mx + logf(sum) : -CUDART_INF_F;
-    }
+  if (grouped) {
     // top-group pruning: only the top_groups live groups by m (ties to the
     // lower group index) keep their experts and their share of p_group
-    if (top_groups > 0 && top_groups < ng) {
+    if (p.top_groups > 0 && p.top_groups < ng) {
       uint32_t keep = 0;
 #pragma unroll 1
       for (int g = 0; g < ng; ++g) {
         if (G[g] == -CUDART_INF_F) continue;
-        const float mg = L[E + g];
+        const float mg = L[p.E + g];
         int rank = 0;
 #pragma unroll 1
         for (int j = 0; j < ng; ++j) {
-          const float mj = L[E + j];
+          const float mj = L[p.E + j];
           if (j != g && G[j] > -CUDART_INF_F && (mj > mg || (mj == mg && j < g))) ++rank;
         }
-        if (rank < top_groups) keep |= 1u << g;
+        if (rank < p.top_groups) keep |= 1u << g;
       }
 #pragma unroll 1
       for (int g = 0; g < ng; ++g)
         if (!((keep >> g) & 1u)) G[g] = -CUDART_INF_F;
     }
-#pragma unroll 1
-    for (int g = 0; g < ng; ++g)
-      if (G[g] > -CUDART_INF_F) mxm = fmaxf(mxm, L[E + g]);
-    float summ = 0.0f;
-#pragma unroll 1
-    for (int g = 0; g < K; ++g)
-      if (G[g] > -CUDART_INF_F) summ += expf(L[E + g] - mxm);
-    lse_m = mxm + logf(summ);
-#pragma unroll 1
-    for (int g = 0; g < ng; ++g) {
-      const float lg = G[g];
-      if (lg == -CUDART_INF_F) continue;  // no allowed member, or pruned
-      const float mk = L[E + g];
-      const int lo = g * gsize, hi = lo + gsize;
+    float mxm = -CUDART_INF_F;
 #pragma unroll 2
-      for (int e = lo; e < hi; ++e) {
-        const float le = L[e];
-        const float key = (mk - lg) + le;
-        if (m.has(e) && key > tk[KS - 1]) topk_insert<KS>(tk, tl, ti, key, e, (mk - lse_m) + (le - lg));
-      }
+    for (int g = 0; g < ng; ++g)
+      if (G[g] > -CUDART_INF_F) mxm = fmaxf(mxm, L[p.E + g]);
+    float summ = 0.0f;
+#pragma unroll 2
+    for (int g = 0; g < ng; ++g)
+      if (G[g] > -CUDART_INF_F) summ += expf(L[p.E + g] - mxm);
+    lse_m = mxm + logf(summ);
+  }
+#pragma unroll 1
+  for (int g = 0; g < ng; ++g) {
+    const float lg = G[g];
+    if (grouped && lg == -CUDART_INF_F) continue;  // no allowed member, or pruned
+    const float mk = grouped ? L[p.E + g] : 0.0f;
+    const int hi = s_grp[g + 1];
+#pragma unroll 2
+    for (int j = s_grp[g]; j < hi; ++j) {
+      const int e = s_list[j];
+      const float le = L[e];
+      const float key = grouped ? (mk - lg) + le : le;
+      if (key > tk[KS - 1]) topk_insert<KS>(tk, tl, ti, key, e, grouped ? (mk - lse_m) + (le - lg) : le - lg);
     }
   }
   // non-finite keys: fill empty slots with the lowest allowed experts not chosen
-  int next = 0;
+  if (ti[KS - 1] < 0) {
+    const MaskRegs m{p.mask_bits[0], p.mask_bits[1], p.mask_bits[2], p.mask_bits[3]};
+    const int gsize = p.E / ng;
+    int next = 0;
 #pragma unroll
-  for (int s = 0; s < KS; ++s) {
-    if (s < k && ti[s] < 0) {
+    for (int s = 0; s < KS; ++s) {
+      if (s < k && ti[s] < 0) {
 #pragma unroll 1
-      for (; next < E; ++next) {
-        if (!m.has(next)) continue;
-        bool used = false;
+        for (; next < p.E; ++next) {
+          if (!m.has(next)) continue;
+          bool used = false;
 #pragma unroll
-        for (int q = 0; q < KS; ++q) used |= (ti[q] == next);
-        if (!used) break;
+          for (int q = 0; q < KS; ++q) used |= (ti[q] == next);
+          if (!used) break;
+        }
+        const int e = next < p.E ? next : 0;
+        ++next;
+        const int g = e / gsize;
+        ti[s] = e;
+        tl[s] = grouped ? (L[p.E + g] - lse_m) + (L[e] - G[g]) : L[e] - G[0];
       }
-      const int e = next < E ? next : 0;
-      ++next;
-      const int g = e / gsize;
-      ti[s] = e;
-      tl[s] = grouped ? (L[E + g] - lse_m) + (L[e] - G[g]) : L[e] - G[0];
     }
   }
   float gw[KS];
@@ -263,86 +268,16 @@ __device__ void decide_token_thread(int E, int K, int k, int renorm, int top_gro
     gw[s] = s < k ? expf(tl[s]) : 0.0f;
     wsum += gw[s];
   }
-#pragma unroll
-  for (int s = 0; s < KS; ++s)
-    if (s < k) {
-      topk_idx[(size_t)tok * k + s] = ti[s];
-      topk_w[(size_t)tok * k + s] = renorm ? gw[s] / wsum : gw[s];
-      if (s_idx) s_idx[s] = ti[s];
-    }
-}
-
-// The same decision for K = 1 from the logits in registers (x[o] for o < E,
-// bias included), fully unrolled so the mask tests are compile-time bit
-// selects and the exponentials are independent: key = l_i, weight
-// exp(l_i - lse) with lse the log-sum-exp of the allowed logits.
-template <int NB, int KS>
-__device__ __forceinline__ void decide_k1_regs(const float (&x)[NB][16], int E, int k, int renorm, const MaskRegs m,
-                                               int32_t* topk_idx, float* topk_w, int tok, int* s_idx) {
-  float tk[KS], tl[KS];
-  int ti[KS];
-#pragma unroll
-  for (int j = 0; j < KS; ++j) {
-    tk[j] = -CUDART_INF_F;
-    tl[j] = 0.0f;
-    ti[j] = -1;
-  }
-  float mx = -CUDART_INF_F;
-#pragma unroll
-  for (int b = 0; b < NB; ++b)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int e = b * 16 + j;
-      if (e < E && m.has(e)) {
-        mx = fmaxf(mx, x[b][j]);
-        if (x[b][j] > tk[KS - 1]) topk_insert<KS>(tk, tl, ti, x[b][j], e, x[b][j]);
-      }
-    }
-  float sum = 0.0f;
-#pragma unroll
-  for (int b = 0; b < NB; ++b)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int e = b * 16 + j;
-      if (e < E && m.has(e)) sum += expf(x[b][j] - mx);
-    }
-  const float lse = mx + logf(sum);
-  // non-finite logits: fill empty slots with the lowest allowed experts not chosen
-#pragma unroll
-  for (int s = 0; s < KS; ++s) {
-    if (s < k && ti[s] < 0) {
-      int pick = -1;
-      float lp = 0.0f;
-#pragma unroll
-      for (int b = NB - 1; b >= 0; --b)
-#pragma unroll
-        for (int j = 15; j >= 0; --j) {
-          const int e = b * 16 + j;
-          bool used = false;
-#pragma unroll
-          for (int q = 0; q < KS; ++q) used |= (ti[q] == e);
-          if (e < E && m.has(e) && !used) {
-            pick = e;
-            lp = x[b][j];
-          }
-        }
-      ti[s] = pick < 0 ? 0 : pick;
-      tl[s] = lp;
-    }
-  }
-  float gw[KS];
-  float wsum = 0.0f;
-#pragma unroll
-  for (int s = 0; s < KS; ++s) {
-    gw[s] = s < k ? expf(tl[s] - lse) : 0.0f;
-    wsum += gw[s];
+  if (!real) {
+    G[0] = wsum;  // keep the work
+    return;
   }
 #pragma unroll
   for (int s = 0; s < KS; ++s)
     if (s < k) {
-      topk_idx[(size_t)tok * k + s] = ti[s];
-      topk_w[(size_t)tok * k + s] = renorm ? gw[s] / wsum : gw[s];
-      if (s_idx) s_idx[s] = ti[s];
+      p.topk_idx[(size_t)tok * k + s] = ti[s];
+      p.topk_w[(size_t)tok * k + s] = p.renorm ? gw[s] / wsum : gw[s];
+      s_idx[s] = ti[s];
     }
 }
 
@@ -447,7 +382,7 @@ __global__ void __launch_bounds__(256) gate_split_kernel(const float* W_local, c
 template <int NB, bool PREP>
 __global__ void __launch_bounds__(GC_THREADS, 1)
     gate_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                   const __grid_constant__ CUtensorMap tmWg, const __grid_constant__ GcParams gp) {
+                   const __grid_constant__ GcParams gp) {
   using namespace tc;
   const KParams& p = gp.kp;
   extern __shared__ uint8_t smem_raw[];
@@ -455,13 +390,15 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
   const int nglob = (p.K == 1) ? 0 : p.K;
   const int O = p.E + nglob;
   const int cs = gp.cs;
-  const GcLayout L(O, p.k, p.E, gp.stages, PREP, cs);
+  const GcLayout L(O, p.k, p.E, gp.stages, cs);
   const int S = gp.stages;
   float* sLog = reinterpret_cast<float*>(smem + L.log_off);
   int* sIdx = reinterpret_cast<int*>(smem + L.idx_off);
   int* sTab = reinterpret_cast<int*>(smem + L.tab_off);
   int* s_base = reinterpret_cast<int*>(smem + L.base_off);
   float* s_bias = reinterpret_cast<float*>(smem + L.bias_off);
+  int* s_list = reinterpret_cast<int*>(smem + L.list_off);
+  int* s_grp = s_list + p.E;
   float* s_recv = reinterpret_cast<float*>(smem + L.recv_off);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L.bar_off);
   uint64_t* conv = full + S;
@@ -509,10 +446,23 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
   }
   for (int o = threadIdx.x - 64; o >= 0 && o < O; o += GC_THREADS - 64)
     s_bias[o] = o < p.E ? p.b_local[o] : p.b_global[o - p.E];
+  if (warp == 2) {
+    // the allowed experts in ascending order, and where each group's begin
+    const int gsize = p.E / p.K;
+    int base = 0;
+    for (int c = 0; c * 32 < p.E; ++c) {
+      const uint32_t bits = p.mask_bits[c];
+      const int e = c * 32 + lane;
+      const int at = base + __popc(bits & ((1u << lane) - 1u));
+      if (bits >> lane & 1u) s_list[at] = e;
+      if (e < p.E && e % gsize == 0) s_grp[e / gsize] = at;
+      base += __popc(bits);
+    }
+    if (lane == 0) s_grp[p.K] = base;
+  }
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmX);
-    tma_prefetch_desc(&tmW);
-    if (!PREP && nglob) tma_prefetch_desc(&tmWg);
+    if (PREP) tma_prefetch_desc(&tmW);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -532,44 +482,46 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
     // Activations do not depend on the previous kernel, the prepared split
     // rows (PREP) do: the X boxes of the first stages go out before the
     // dependency wait, their split rows after it.
-    if (lane == 0) {
-      const uint32_t xbytes = GC_BM * GC_BK * 2;
-      const uint32_t wbytes = PREP ? 3 * n_pad * GC_BK * 2 : O * GC_BK * 4;
+    // The whole warp waits and counts; one elected lane issues.
+    {
+      const bool issue = elect_one();
+      const uint32_t bytes = GC_BM * GC_BK * 2 + (PREP ? 3 * n_pad * GC_BK * 2 : 0);
       const int my_tiles = tile_first < n_tiles ? (n_tiles - 1 - tile_first) / tile_step + 1 : 0;
       const int total = my_tiles * cnt;
-      const int pre = PREP ? (total < S ? total : S) : 0;
-      auto load_w = [&](int c, uint8_t* st, uint32_t fb) {
-        const int kc = kb_lo + c % cnt;
-        if (PREP) {
-          tma_load_2d(smem_u32(st + L.w3_off), &tmW, kc * GC_BK, 0, fb);
-        } else {
-          tma_load_2d(smem_u32(st + L.raw_off), &tmW, kc * GC_BK, 0, fb);
-          if (nglob) tma_load_2d(smem_u32(st + L.raw_off + p.E * GC_BK * 4), &tmWg, kc * GC_BK, 0, fb);
+      const int pre = total < S ? total : S;
+      int kc = 0, x_row = tile_first * GC_BM;  // next stage's place
+      auto load_x = [&](uint8_t* st, uint32_t fb) {
+        if (issue) {
+          mbar_expect_tx(fb, bytes);
+          tma_load_2d(smem_u32(st), &tmX, (kb_lo + kc) * GC_BK, x_row, fb);
         }
       };
-      for (int c = 0; c < pre; ++c) {
-        const uint32_t fb = smem_u32(&full[c]);
-        mbar_expect_tx(fb, xbytes + wbytes);
-        tma_load_2d(smem_u32(smem + c * L.stage_bytes), &tmX, (kb_lo + c % cnt) * GC_BK,
-                    (tile_first + (c / cnt) * tile_step) * GC_BM, fb);
-      }
+      auto next = [&] {
+        if (++kc == cnt) {
+          kc = 0;
+          x_row += tile_step * GC_BM;
+        }
+      };
+      for (int c = 0; c < pre; ++c, next()) load_x(smem + c * L.stage_bytes, smem_u32(&full[c]));
       pdl_wait();
-      for (int c = 0; c < pre; ++c) load_w(c, smem + c * L.stage_bytes, smem_u32(&full[c]));
-      int stage = pre % S;
+      if (PREP && issue)
+        for (int c = 0, wk = 0; c < pre; ++c, wk = wk + 1 == cnt ? 0 : wk + 1)
+          tma_load_2d(smem_u32(smem + c * L.stage_bytes + L.w3_off), &tmW, (kb_lo + wk) * GC_BK, 0, smem_u32(&full[c]));
+      int stage = pre == S ? 0 : pre;
       uint32_t phase = (pre == S) ? 1u : 0u;
       uint32_t issued = pre ? ((1u << pre) - 1u) : 0u, issued_phase = 0;
       bool ok = true;
       for (int c = pre; c < total; ++c) {
-        if (!mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_gate_error)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_gate_error))) {
           ok = false;
           break;
         }
         uint8_t* st = smem + stage * L.stage_bytes;
         const uint32_t fb = smem_u32(&full[stage]);
-        mbar_expect_tx(fb, xbytes + wbytes);
-        tma_load_2d(smem_u32(st), &tmX, (kb_lo + c % cnt) * GC_BK, (tile_first + (c / cnt) * tile_step) * GC_BM,
-                    fb);
-        load_w(c, st, fb);
+        load_x(st, fb);
+        if (PREP && issue) tma_load_2d(smem_u32(st + L.w3_off), &tmW, (kb_lo + kc) * GC_BK, 0, fb);
+        next();
         issued |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
         if (++stage == S) {
@@ -643,13 +595,25 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
     }
   } else {
     // ------------------------------------------------------------ worker warps
-    pdl_wait();  // the routing counters are cleared by the previous kernel (PREP)
     const int wt = threadIdx.x - 64;
     const bool is_drain = warp < 6;
     const int q = warp & 3;
     const int row = q * 32 + lane;
     const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-    const MaskRegs mregs{p.mask_bits[0], p.mask_bits[1], p.mask_bits[2], p.mask_bits[3]};
+    auto pick = [&](float* Lr, int* sx, int tok, bool real) {
+      if (p.k == 1) pick_row<1>(p, Lr, O, s_list, s_grp, tok, sx, real);
+      else if (p.k == 2) pick_row<2>(p, Lr, O, s_list, s_grp, tok, sx, real);
+      else if (p.k <= 4) pick_row<4>(p, Lr, O, s_list, s_grp, tok, sx, real);
+      else pick_row<8>(p, Lr, O, s_list, s_grp, tok, sx, real);
+    };
+    if (PREP && warp == 6) {
+      // an idle warp: bring the decision's code to the SM (on a row of its own,
+      // whatever it holds; nothing reads the outcome)
+      float* warm = reinterpret_cast<float*>(smem + L.warm_off);
+      lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
+      pick(warm, nullptr, 0, false);
+    }
+    pdl_wait();  // the routing counters are cleared by the previous kernel (PREP)
     int stage = 0;
     uint32_t phase = 0;
     int acc_sel = 0;
@@ -722,62 +686,53 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
           }
         }
         if (decide_here) {
+          float* Lrow = sLog + row * L.log_stride;
 #pragma unroll
           for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int o = b * 16 + j;
-              if (o < O) acc[b][j] += s_bias[o];
+              if (o < O) Lrow[o] = acc[b][j] + s_bias[o];
             }
-          const int tok = tile * GC_BM + row;
-          int* sx = p.route_counts ? sIdx + row * p.k : nullptr;
           if (!nglob) {
-            if (tok < p.T) {
-              if (p.k == 1) decide_k1_regs<NB, 1>(acc, p.E, p.k, p.renorm, mregs, p.topk_idx, p.topk_w, tok, sx);
-              else if (p.k == 2) decide_k1_regs<NB, 2>(acc, p.E, p.k, p.renorm, mregs, p.topk_idx, p.topk_w, tok, sx);
-              else if (p.k <= 4) decide_k1_regs<NB, 4>(acc, p.E, p.k, p.renorm, mregs, p.topk_idx, p.topk_w, tok, sx);
-              else decide_k1_regs<NB, 8>(acc, p.E, p.k, p.renorm, mregs, p.topk_idx, p.topk_w, tok, sx);
-            }
-          } else {
-            float* Lrow = sLog + row * L.log_stride;
+            // one group: the row's own thread takes the whole decision
+            const int tok = tile * GC_BM + row;
+            lse_rows(sLog, L.log_stride, O, s_list, s_grp, 1, row, 1, 0, 1);
+            if (tok < p.T) pick(Lrow, sIdx + row * p.k, tok, true);
+          }
+        }
+      } else if (!PREP) {
+        // split the fp32 gate rows of each stage into three bf16 terms, written
+        // in the swizzled K-major layout of the B operand; the next stage's
+        // pieces (8 columns of a row) are loaded while this one is written
+        const int ct = threadIdx.x - 192;
+        constexpr int ITEMS = (GC_MAX_O * 8 + 255) / 256;
+        float v[ITEMS][8];
+        auto load_items = [&](int kc) {
 #pragma unroll
-            for (int b = 0; b < NB; ++b)
+          for (int t = 0; t < ITEMS; ++t) {
+            const int i = ct + 256 * t, r = i >> 3, c = kc * GC_BK + (i & 7) * 8;
+            if (r < O && c < p.d) {
+              load8((r < p.E ? p.W_local + (size_t)r * p.d : p.W_global + (size_t)(r - p.E) * p.d) + c, v[t]);
+            } else {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const int o = b * 16 + j;
-                if (o < O) Lrow[o] = acc[b][j];
-              }
-            if (tok < p.T) {
-              if (p.k == 1) decide_token_thread<1>(p.E, p.K, p.k, p.renorm, p.top_groups, mregs, Lrow, Lrow + O, p.topk_idx, p.topk_w, tok, sx);
-              else if (p.k == 2) decide_token_thread<2>(p.E, p.K, p.k, p.renorm, p.top_groups, mregs, Lrow, Lrow + O, p.topk_idx, p.topk_w, tok, sx);
-              else if (p.k <= 4) decide_token_thread<4>(p.E, p.K, p.k, p.renorm, p.top_groups, mregs, Lrow, Lrow + O, p.topk_idx, p.topk_w, tok, sx);
-              else decide_token_thread<8>(p.E, p.K, p.k, p.renorm, p.top_groups, mregs, Lrow, Lrow + O, p.topk_idx, p.topk_w, tok, sx);
+              for (int u = 0; u < 8; ++u) v[t][u] = 0.0f;
             }
           }
-        }  // decide_here
-      } else if (!PREP) {
-        // split the raw fp32 gate rows of each stage into three bf16 terms,
-        // written in the swizzled K-major layout of the B operand
-        const int ct = threadIdx.x - 192;
+        };
+        load_items(kb_lo);
         for (int kc = 0; kc < cnt; ++kc) {
-          if (ok) ok = mbar_wait(smem_u32(&full[stage]), phase, budget, abort_flag, &g_gate_error);
+          if (ok)
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_gate_error));
           if (ok) {
             uint8_t* st = smem + stage * L.stage_bytes;
-            const float* raw = reinterpret_cast<const float*>(st + L.raw_off);
-            for (int i = ct; i < n_pad * 8; i += 256) {
-              const int r = i >> 3, ch = i & 7;
-              float v[8];
-              if (r < O) {
-                const float4 a = *reinterpret_cast<const float4*>(raw + r * GC_BK + ch * 8);
-                const float4 b = *reinterpret_cast<const float4*>(raw + r * GC_BK + ch * 8 + 4);
-                v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-              } else {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = 0.0f;
-              }
+            for (int t = 0; t < ITEMS; ++t) {
+              const int i = ct + 256 * t, r = i >> 3, ch = i & 7;
+              if (r >= n_pad) break;
               uint32_t t0[4], t1[4], t2[4];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) split3_pair(v[2 * u], v[2 * u + 1], t0[u], t1[u], t2[u]);
+              for (int u = 0; u < 4; ++u) split3_pair(v[t][2 * u], v[t][2 * u + 1], t0[u], t1[u], t2[u]);
               const int off = L.w3_off + r * 128 + ((ch ^ (r & 7)) << 4);
               *reinterpret_cast<U4*>(st + off) = U4{t0[0], t0[1], t0[2], t0[3]};
               *reinterpret_cast<U4*>(st + off + n_pad * 128) = U4{t1[0], t1[1], t1[2], t1[3]};
@@ -788,11 +743,27 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&conv[stage]));
+          if (kc + 1 < cnt) load_items(kb_lo + kc + 1);
           if (++stage == S) {
             stage = 0;
             phase ^= 1u;
           }
         }
+      }
+      // the tile's decisions over several groups: all worker warps (without
+      // prepared rows the drain warps alone, while the others convert the next
+      // tile's rows)
+      const int n_dec = PREP ? GC_WORKERS : 128;
+      const int first_row = rank * rows_own;
+      if (nglob && (PREP || is_drain)) {
+        asm volatile("bar.sync 2, %0;" ::"r"(n_dec) : "memory");
+        lse_rows(sLog, L.log_stride, O, s_list, s_grp, p.K, first_row, rows_own, wt, n_dec);
+        asm volatile("bar.sync 2, %0;" ::"r"(n_dec) : "memory");
+        const int tok = tile * GC_BM + first_row + wt;
+        const int r = first_row + wt;
+        if (wt < rows_own && tok < p.T) pick(sLog + r * L.log_stride, sIdx + r * p.k, tok, true);
+        // the rows are read before the next tile's logits replace them
+        if (!p.route_counts) asm volatile("bar.sync 2, %0;" ::"r"(n_dec) : "memory");
       }
       if (p.route_counts) {
         asm volatile("bar.sync 1, %0;" ::"r"(GC_WORKERS) : "memory");
@@ -813,17 +784,18 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
 }
 
 // Stages that fit next to the logits, routing tables and received partials.
-int gc_stages(int O, int k, int E, bool prep, int cs) {
+int gc_stages(int O, int k, int E, int cs) {
   for (int s = GC_MAX_STAGES; s >= 2; --s)
-    if (GcLayout(O, k, E, s, prep, cs).total + 1024 <= 232448) return s;
+    if (GcLayout(O, k, E, s, cs).total + 1024 <= 232448) return s;
   return 0;
 }
 
 // CTAs per tile: d_model is split over a cluster of GC_CS when a tile has at
-// least GC_SPLIT_MIN_NK stages and the received partials still leave four
-// pipeline stages (counted for the larger, self-splitting layout), whatever
-// the token count and whether the rows come prepared, so every call of one
-// layer shape sums its logits in the same order.
+// least GC_SPLIT_MIN_NK stages and the received partials still leave room for
+// four stages that hold the fp32 gate rows as well (more gate rows make the
+// exchange too large a part), whatever the token count and whether the rows
+// come prepared, so every call of one layer shape sums its logits in the same
+// order.
 // EC2MOE_GATE_SPLIT_MIN_STAGES=n in the environment moves the threshold
 // (A/B comparisons; the split computes the same logits up to summation order).
 int gc_cluster_size(int O, int k, int E, int d) {
@@ -832,7 +804,8 @@ int gc_cluster_size(int O, int k, int E, int d) {
     return v && atoi(v) > 0 ? atoi(v) : GC_SPLIT_MIN_NK;
   }();
   if ((d + GC_BK - 1) / GC_BK < min_nk) return 1;
-  return gc_stages(O, k, E, false, GC_CS) >= 4 ? GC_CS : 1;
+  const GcLayout four(O, k, E, 4, GC_CS);
+  return four.warm_off + 4 * four.n_pad * 256 + 1024 <= 232448 ? GC_CS : 1;
 }
 
 // CTAs the gate kernel launches (cs > 1: a cluster per tile, run in waves
@@ -845,7 +818,7 @@ int gc_blocks(int T, int cs) {
 
 template <int NB, bool PREP>
 cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t s, const CUtensorMap& mX,
-                              const CUtensorMap& mW, const CUtensorMap& mWg) {
+                              const CUtensorMap& mW) {
   const int O = p.E + (p.K == 1 ? 0 : p.K);
   GcParams gp;
   gp.kp = p;
@@ -853,12 +826,12 @@ cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t
   gp.stages = stages;
   gp.cs = cs;
   gp.timeout = default_timeout_cycles();
-  const int smem = GcLayout(O, p.k, p.E, stages, PREP, cs).total + 1024;
+  const int smem = GcLayout(O, p.k, p.E, stages, cs).total + 1024;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(gate_tc_kernel<NB, PREP>), smem);
   if (e != cudaSuccess) return e;
   const int blocks = gc_blocks(p.T, cs);
   if (cs == 1)
-    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(GC_THREADS), (size_t)smem, s, mX, mW, mWg, gp);
+    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(GC_THREADS), (size_t)smem, s, mX, mW, gp);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(GC_THREADS);
@@ -873,20 +846,20 @@ cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = next_launch_pdl() ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gate_tc_kernel<NB, PREP>, mX, mW, mWg, gp);
+  return cudaLaunchKernelEx(&cfg, gate_tc_kernel<NB, PREP>, mX, mW, gp);
 }
 
 template <bool PREP>
 cudaError_t launch_gate_tc(const KParams& p, int stages, int cs, cudaStream_t s, const CUtensorMap& mX,
-                           const CUtensorMap& mW, const CUtensorMap& mWg) {
+                           const CUtensorMap& mW) {
   const int O = p.E + (p.K == 1 ? 0 : p.K);
   // NB = accumulator blocks of 16 gate rows a drain thread keeps; 3 and 4
   // run as 5 (the extra blocks read allocated TMEM columns past the gate rows
   // and are never used), which keeps the number of kernel variants small.
   switch ((O + 15) / 16) {
-    case 1: return launch_gate_tc_nb<1, PREP>(p, stages, cs, s, mX, mW, mWg);
-    case 2: return launch_gate_tc_nb<2, PREP>(p, stages, cs, s, mX, mW, mWg);
-    default: return launch_gate_tc_nb<5, PREP>(p, stages, cs, s, mX, mW, mWg);
+    case 1: return launch_gate_tc_nb<1, PREP>(p, stages, cs, s, mX, mW);
+    case 2: return launch_gate_tc_nb<2, PREP>(p, stages, cs, s, mX, mW);
+    default: return launch_gate_tc_nb<5, PREP>(p, stages, cs, s, mX, mW);
   }
 }
 
@@ -910,16 +883,13 @@ cudaError_t launch_gate_tensor(const GateArgs& a, KParams p, int O, bool bf16, c
     const bool prep = a.w_split != nullptr;
     const int n_pad = (O + 15) / 16 * 16;
     const int cs = gc_cluster_size(O, a.k, a.E, a.d);
-    const int stages = gc_stages(O, a.k, a.E, prep, cs);
-    CUtensorMap mX, mW, mWg;
+    const int stages = gc_stages(O, a.k, a.E, cs);
+    CUtensorMap mX, mW;
     bool maps = stages >= 2 && make_tensor_map_bf16(&mX, a.X, a.T, a.d, GC_BM);
     if (prep) {
       maps = maps && make_tensor_map_bf16(&mW, a.w_split, 3LL * n_pad, a.d, 3 * n_pad);
-      mWg = mW;
-    } else {
-      maps = maps && make_tensor_map_f32(&mW, a.W_local, a.E, a.d, a.E);
-      if (maps && a.K > 1) maps = make_tensor_map_f32(&mWg, a.W_global, a.K, a.d, a.K);
-      else mWg = mW;
+    } else if (maps) {
+      mW = mX;  // not read: the kernel loads and splits the gate rows itself
     }
     if (maps) {
       *handled = true;
@@ -946,8 +916,8 @@ cudaError_t launch_gate_tensor(const GateArgs& a, KParams p, int O, bool bf16, c
         const int b = gc_blocks(a.T, cs);
         *held_sms = b < sm_count() ? b : sm_count();
       }
-      e = prep ? launch_gate_tc<true>(p, stages, cs, s, mX, mW, mWg)
-               : launch_gate_tc<false>(p, stages, cs, s, mX, mW, mWg);
+      e = prep ? launch_gate_tc<true>(p, stages, cs, s, mX, mW)
+               : launch_gate_tc<false>(p, stages, cs, s, mX, mW);
       if (e != cudaSuccess) return e;
       return cudaGetLastError();
     }
