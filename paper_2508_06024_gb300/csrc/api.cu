@@ -465,6 +465,8 @@ cudaError_t run_codec(const ec2moe_layer_desc* d, bool encode, const void* in, c
     g.rep_E = d->E;
     return run_gemm(d, g, EPI_REPLICATE, s);
   }
+  // the encoder reads X and V_enc alone: it runs beside the gate before it
+  g.early = encode ? 1 : 0;
   const int split = encode && enc_partial ? enc_split(d) : 1;
   if (split > 1) {
     g.split_k = split;

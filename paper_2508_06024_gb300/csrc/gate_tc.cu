@@ -606,8 +606,9 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
       else if (p.k <= 4) pick_row<4>(p, Lr, O, s_list, s_grp, tok, sx, real);
       else pick_row<8>(p, Lr, O, s_list, s_grp, tok, sx, real);
     };
-    if (PREP && warp == 6) {
-      // an idle warp: bring the decision's code to the SM (on a row of its own,
+    if (warp == (PREP ? 6 : 5)) {
+      // an idle warp (without prepared rows a drain warp, which has nothing to do
+      // before the first segment ends): bring the decision's code to the SM (on a row of its own,
       // whatever it holds; nothing reads the outcome)
       float* warm = reinterpret_cast<float*>(smem + L.warm_off);
       lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);

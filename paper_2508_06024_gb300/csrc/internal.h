@@ -210,6 +210,12 @@ struct GemmArgs {
   float* partial;                    // EPI_PARTIAL: fp32 [split_k][part_rows][N]
   long long part_rows;
   long long timeout_cycles;          // bounded-wait budget (tensor-core path)
+  // launch_gemm_tc: A and B are inputs of the public call and nothing in flight
+  // before this launch touches `out` or `partial`, so the kernel need not wait
+  // for its predecessor before it starts (programmatic dependent launch); it
+  // still ends after it.  The kernels of a call release their successors at
+  // their start, so results of any earlier kernel of the call do not qualify.
+  int early;
   const char* name;                  // label for per-launch profiling (nullptr = by epilogue)
 };
 cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s);    // bf16, tcgen05

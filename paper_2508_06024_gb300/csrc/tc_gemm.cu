@@ -100,6 +100,7 @@ struct Params {
   long long timeout;
   int n_tiles_n;
   int split_k, kb_per_split;
+  int early;  // reads only the call's inputs: wait for the previous kernel at the end, not before
   float* partial;
   long long part_rows;
   long long row_limit;  // rows of the call: group ranges and scatter destinations lie in [0, row_limit)
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 0) {
-    pdl_wait();
+    if (!p.early) pdl_wait();
     // Per-group first rows and tile prefix (m tiles), one warp-wide scan.
     warp_exclusive_scan<(MAX_GROUPS + 31) / 32>(
         p.G, lane,
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   // PAIR: both CTAs' barriers are initialised before either arrives remotely
   if (PAIR) cluster_sync_all();
   tc_fence_after();
-  pdl_wait();
+  if (!p.early) pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
   // Split-K (EPI_PARTIAL): tile t covers output tile t / split_k and the
   // k-blocks [ks * kb_per_split, ...) with ks = t % split_k.
@@ -687,6 +688,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   }
 
+  // An early kernel ends after its predecessor, so that kernels behind it may
+  // rely on both.
+  if (p.early) pdl_wait();
   tc_fence_before();
   __syncthreads();
   // PAIR: the even CTA's MMAs write both CTAs' TMEM; neither releases its
@@ -824,6 +828,7 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   p.rep_offsets_out = a.rep_offsets_out;
   p.rep_E = a.rep_E;
   p.timeout = a.timeout_cycles;
+  p.early = a.early;
   p.n_tiles_n = (a.N + C::BN_OUT - 1) / C::BN_OUT;
   p.split_k = EPI == EPI_PARTIAL && a.split_k > 1 ? a.split_k : 1;
   {
