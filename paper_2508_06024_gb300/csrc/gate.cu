@@ -716,44 +716,52 @@ __global__ void __launch_bounds__(SL_THREADS) gate_tiled_kernel(const KParams p)
 
 // ---- small batches (T <= 256): the d_model axis split across CTAs
 // One or two 128-token tiles leave a per-tile kernel with one or two CTAs
-// walking all of d_model.  Here CTA (c, b) takes the GP_DC columns of chunk c
-// for the GP_TB tokens of tile b: it stages the gate-row slice (fp32) and the
-// activation slice (as fp32) in shared memory and writes the fp32 partial
-// logits of its chunk; a second kernel adds the chunks in chunk order, adds
+// walking all of d_model.  Here CTA (c, b, z) takes the GP_DC columns of chunk c
+// for the GP_TB tokens of tile b and the GP_RO gate rows of slice z: it stages
+// the gate-row slice (fp32) and the activation slice (as fp32) in shared memory
+// and writes the fp32 partial logits of its chunk (loads in a chain bound it:
+// with all 72 gate rows of the fine-grained layer in one CTA, 16 CTAs took 20.7
+// us launch bracket included); a second kernel adds the chunks in chunk order, adds
 // the bias, and takes the same warp decision and in-kernel routing as the
 // other gates.  Partials: [n_chunks][T][O].
 constexpr int GP_TB = 64;
 constexpr int GP_DC = 128;
 constexpr int GP_PITCH = GP_DC + 4;  // floats; rows 16-byte aligned, float4 reads of 8 rows on distinct banks
 constexpr int GP_OB = 8;
+constexpr int GP_RO = 24;            // gate rows per CTA: one item per thread
 constexpr int GP_THREADS = 256;
-constexpr int GD_BT = 8;             // tokens per CTA of the decision kernel (one warp each)
+constexpr int GD_BT = 8;             // most tokens per CTA of the decision kernel (one warp each)
+constexpr int GD_BT_PLAIN = 2;       // without the weight prefetch: fewer sums per CTA in a row
 
-size_t gp_smem(int O) { return (size_t)(O + GP_TB) * GP_PITCH * sizeof(float); }
+size_t gp_smem(int O) { return (size_t)((O < GP_RO ? O : GP_RO) + GP_TB) * GP_PITCH * sizeof(float); }
 
 template <typename TX>
 __global__ void __launch_bounds__(GP_THREADS) gate_partial_kernel(const KParams p, float* __restrict__ part) {
   extern __shared__ float4 gp_smem_v[];
-  float* sW = reinterpret_cast<float*>(gp_smem_v);  // [O][GP_PITCH]
+  float* sW = reinterpret_cast<float*>(gp_smem_v);  // [n_o][GP_PITCH]
   const int O = p.E + (p.K == 1 ? 0 : p.K);
-  float* sX = sW + (size_t)O * GP_PITCH;            // [GP_TB][GP_PITCH]
+  const int o0 = blockIdx.z * GP_RO;                // this CTA's gate rows [o0, o0 + n_o)
+  const int n_o = O - o0 < GP_RO ? O - o0 : GP_RO;
+  float* sX = sW + (size_t)n_o * GP_PITCH;          // [GP_TB][GP_PITCH]
   const int c0 = blockIdx.x * GP_DC;
   const int t0 = blockIdx.y * GP_TB;
   pdl_trigger();
   // gate-row slice: constant weights, staged before waiting on the previous kernel
-  for (int i = threadIdx.x; i < O * (GP_DC / 4); i += GP_THREADS) {
-    const int o = i / (GP_DC / 4), c = (i % (GP_DC / 4)) * 4;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n_o * (GP_DC / 4); i += GP_THREADS) {
+    const int o = o0 + i / (GP_DC / 4), c = (i % (GP_DC / 4)) * 4;
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (c0 + c < p.d) {
       const float* row = o < p.E ? p.W_local + (size_t)o * p.d : p.W_global + (size_t)(o - p.E) * p.d;
       v = *reinterpret_cast<const float4*>(row + c0 + c);
     }
-    *reinterpret_cast<float4*>(sW + o * GP_PITCH + c) = v;
+    *reinterpret_cast<float4*>(sW + (o - o0) * GP_PITCH + c) = v;
   }
   pdl_wait();
-  if (p.route_counts && blockIdx.x == 0 && blockIdx.y == 0)
+  if (p.route_counts && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
     for (int e = threadIdx.x; e < p.E; e += GP_THREADS) p.route_counts[e] = 0;
   const TX* X = reinterpret_cast<const TX*>(p.X);
+#pragma unroll
   for (int i = threadIdx.x; i < GP_TB * (GP_DC / 8); i += GP_THREADS) {
     const int t = i / (GP_DC / 8), c = (i % (GP_DC / 8)) * 8;
     float f[8];
@@ -767,7 +775,7 @@ __global__ void __launch_bounds__(GP_THREADS) gate_partial_kernel(const KParams 
   __syncthreads();
   // item = (token t, block of GP_OB gate rows); lanes run over tokens so the
   // gate-row reads are warp broadcasts
-  const int nob = (O + GP_OB - 1) / GP_OB;
+  const int nob = (n_o + GP_OB - 1) / GP_OB;
   for (int item = threadIdx.x; item < GP_TB * nob; item += GP_THREADS) {
     const int t = item % GP_TB, ob = item / GP_TB;
     const int tok = t0 + t;
@@ -781,7 +789,7 @@ __global__ void __launch_bounds__(GP_THREADS) gate_partial_kernel(const KParams 
       const float4 xv = *reinterpret_cast<const float4*>(xr + c);
 #pragma unroll
       for (int j = 0; j < GP_OB; ++j) {
-        const int o = ob * GP_OB + j < O ? ob * GP_OB + j : O - 1;  // clamped read, result unused
+        const int o = ob * GP_OB + j < n_o ? ob * GP_OB + j : n_o - 1;  // clamped read, result unused
         const float4 wv = *reinterpret_cast<const float4*>(sW + o * GP_PITCH + c);
         acc[j] = fmaf(xv.x, wv.x, acc[j]);
         acc[j] = fmaf(xv.y, wv.y, acc[j]);
@@ -789,14 +797,14 @@ __global__ void __launch_bounds__(GP_THREADS) gate_partial_kernel(const KParams 
         acc[j] = fmaf(xv.w, wv.w, acc[j]);
       }
     }
-    float* dst = part + ((size_t)blockIdx.x * p.T + tok) * O;
+    float* dst = part + ((size_t)blockIdx.x * p.T + tok) * O + o0;
 #pragma unroll
     for (int j = 0; j < GP_OB; ++j)
-      if (ob * GP_OB + j < O) dst[ob * GP_OB + j] = acc[j];
+      if (ob * GP_OB + j < n_o) dst[ob * GP_OB + j] = acc[j];
   }
 }
 
-// Decision kernel: GD_BT tokens per CTA (one warp each).  The chunk sums are
+// Decision kernel: bt <= GD_BT tokens per CTA (one warp each).  The chunk sums are
 // split four ways (group g adds chunks g, g + 4, ... in order; then the four
 // group sums are added in group order), so each thread keeps eight loads in
 // flight and the result does not depend on the launch.
@@ -807,13 +815,13 @@ __global__ void __launch_bounds__(GP_THREADS) gate_partial_kernel(const KParams 
 // idle during the codec kernels that follow fills L2 with weights.
 constexpr int GD_SPLIT = 4;
 __global__ void __launch_bounds__(SL_THREADS) gate_decide_kernel(const KParams p, const float* __restrict__ part,
-                                                                 int n_chunks) {
+                                                                 int n_chunks, int bt) {
   extern __shared__ float4 gd_smem_v[];
   const int O = p.E + (p.K == 1 ? 0 : p.K);
-  const int pairs = GD_BT * O;
-  float* sLog = reinterpret_cast<float*>(gd_smem_v);                  // [GD_BT][O]
-  float* sGrp = sLog + pairs;                                          // [GD_SPLIT][GD_BT * O]
-  int* sIdx = reinterpret_cast<int*>(sGrp + GD_SPLIT * pairs);        // [GD_BT * k]
+  const int pairs = bt * O;
+  float* sLog = reinterpret_cast<float*>(gd_smem_v);                  // [bt][O]
+  float* sGrp = sLog + pairs;                                          // [GD_SPLIT][bt * O]
+  int* sIdx = reinterpret_cast<int*>(sGrp + GD_SPLIT * pairs);        // [bt * k]
   __shared__ int s_base[128];
   __shared__ int s_active[129];  // prefetch: chosen experts in id order, then their count
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -825,7 +833,7 @@ __global__ void __launch_bounds__(SL_THREADS) gate_decide_kernel(const KParams p
   const size_t plane = (size_t)p.T * O;
   for (int i = threadIdx.x; i < GD_SPLIT * pairs; i += SL_THREADS) {
     const int g = i / pairs, pr = i % pairs;
-    const int tok = tile * GD_BT + pr / O;
+    const int tok = tile * bt + pr / O;
     float sum = 0.0f;
     if (tok < p.T) {
       const float* src = part + (size_t)tok * O + pr % O;
@@ -851,13 +859,13 @@ __global__ void __launch_bounds__(SL_THREADS) gate_decide_kernel(const KParams p
     sLog[pr] = sum + (o < p.E ? p.b_local[o] : p.b_global[o - p.E]);
   }
   __syncthreads();
-  for (int jj = warp; jj < GD_BT; jj += SL_THREADS / 32) {
-    const int tok = tile * GD_BT + jj;
+  for (int jj = warp; jj < bt; jj += SL_THREADS / 32) {
+    const int tok = tile * bt + jj;
     if (tok < p.T)
       decide_token_warp(p, sLog + jj * O, tok, lane, (p.route_counts || pf) ? sIdx + jj * p.k : nullptr, writer);
   }
   __syncthreads();
-  if (writer && p.route_counts) route_tile(p, tile, GD_BT, sIdx, s_base);
+  if (writer && p.route_counts) route_tile(p, tile, bt, sIdx, s_base);
   if (!pf) return;
   // the chosen experts in id order (the swapped GEMM's active groups)
   if (warp == 0) {
@@ -912,18 +920,19 @@ cudaError_t launch_gate_partial(const GateArgs& a, const KParams& p, int O, cuda
   if (e != cudaSuccess) return e;
   {
     KernelScope ks("gate_topk", s);
-    e = launch_kernel(gate_partial_kernel<TX>, dim3(n_chunks, (a.T + GP_TB - 1) / GP_TB), dim3(GP_THREADS),
+    e = launch_kernel(gate_partial_kernel<TX>, dim3(n_chunks, (a.T + GP_TB - 1) / GP_TB, (O + GP_RO - 1) / GP_RO), dim3(GP_THREADS),
                       (size_t)smem_a, s, p, a.gate_partial);
     if (e != cudaSuccess) return e;
   }
-  const int smem_b = (GD_BT * O * (1 + GD_SPLIT) + GD_BT * a.k) * 4;
+  const int bt = p.pf_w1 ? GD_BT : GD_BT_PLAIN;
+  const int smem_b = (bt * O * (1 + GD_SPLIT) + bt * a.k) * 4;
   e = ensure_smem_attr(reinterpret_cast<const void*>(gate_decide_kernel), smem_b);
   if (e != cudaSuccess) return e;
   KernelScope ks("gate_decide", s);
   // with the prefetch: one CTA per swapped-GEMM CTA, all on the one tile
-  const int blocks = p.pf_w1 ? a.pf_units : (a.T + GD_BT - 1) / GD_BT;
+  const int blocks = p.pf_w1 ? a.pf_units : (a.T + bt - 1) / bt;
   e = launch_kernel(gate_decide_kernel, dim3(blocks), dim3(SL_THREADS), (size_t)smem_b, s, p,
-                    static_cast<const float*>(a.gate_partial), n_chunks);
+                    static_cast<const float*>(a.gate_partial), n_chunks, bt);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -978,7 +987,7 @@ cudaError_t launch_gate(const GateArgs& a, bool bf16, cudaStream_t s, bool* rout
       p.pf_tile_rows = a.pf_tile_rows;
       p.pf_row_bytes = a.pf_row_bytes;
     }
-    if (held_sms) *held_sms = (a.T + GD_BT - 1) / GD_BT;
+    if (held_sms) *held_sms = (a.T + GD_BT_PLAIN - 1) / GD_BT_PLAIN;
     return bf16 ? launch_gate_partial<__nv_bfloat16>(a, p, O, s) : launch_gate_partial<float>(a, p, O, s);
   }
   {
