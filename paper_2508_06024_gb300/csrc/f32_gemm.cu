@@ -97,11 +97,13 @@ struct FCfg {
   static constexpr int OFF_ROW0 = OFF_PREFIX + (MAX_GROUPS + 1) * 4;
   static constexpr int SMEM = 1024 + OFF_ROW0 + MAX_GROUPS * 4;
   static constexpr int TMEM_COLS = 4 * BN;  // two pairs of accumulators
-  static constexpr int NC = BN / 4;         // accumulator columns of a worker thread
+  static constexpr int NC = BN / 4;         // accumulator columns of a thread
+  static constexpr int PITCH = BN + 4;      // floats per row of the result tile (conflict-free 16-byte columns)
   static constexpr int A_CHUNKS = BM * BK / 4 / NUM_THREADS;  // 16-byte pieces per thread and block
   static constexpr int B_CHUNKS = BN * BK / 4 / NUM_THREADS;
   static_assert(SMEM <= 232448 && OFF_BARS % 1024 == 0, "shared memory per CTA");
   static_assert((MAX_SPLIT - 1) * NUM_THREADS * NC * 4 <= STAGES * STAGE_BYTES, "the other CTAs' sums fit the stages");
+  static_assert(BM * PITCH * 4 <= STAGES * STAGE_BYTES, "the result tile fits the stages");
   static_assert(TMEM_COLS == 256 || TMEM_COLS == 512, "TMEM allocation");
 };
 
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* tile_prefix = reinterpret_cast<int*>(smem + C::OFF_PREFIX);
   int* row0 = reinterpret_cast<int*>(smem + C::OFF_ROW0);
+  float* tile_out = reinterpret_cast<float*>(smem);  // the result tile, over the stages
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   pdl_trigger();
@@ -447,65 +450,66 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
             acc[j + 3] += o.w;
           }
         }
-        // every read is done before the next tile's blocks overwrite the sums
+        // every read is done before the result tile below overwrites the sums
         asm volatile("bar.sync 1, %0;" ::"r"(NUM_THREADS) : "memory");
       }
-      if (!ok) continue;
 
-      // epilogue: this thread's row, NC columns in two runs
-      const int local = q * 32 + lane;
-      if (local >= m_left) continue;
-      const long long out_row = p.out_row_base + row0[tc.g] + (long long)tc.m_blk * BM + local;
-      long long dest = out_row;
-      float sc = 1.0f;
-      if (EPI == EPI_SCATTER) {
-        dest = p.perm ? p.perm[out_row] : out_row;
-        if (dest < 0 || dest >= p.row_limit) {
-          atomicOr(&g_f32_error, 2u);
-          continue;
-        }
-        if (p.scale) sc = p.scale[dest];
+      // Epilogue through shared memory (the stages are idle until the next
+      // tile): rows of BN + 4 floats, then whole rows back, 16 bytes per thread
+      // in a rolled loop.  Straight from the accumulator registers it was 4-6 KB
+      // of code per variant, run once per tile, and 16-byte pieces of 32 rows
+      // per store.
+      {
+        float* row = tile_out + (q * 32 + lane) * C::PITCH;
+#pragma unroll
+        for (int j = 0; j < NC; j += 4)
+          *reinterpret_cast<float4*>(row + (j < NC / 2 ? c0 + j : c1 + j - NC / 2)) =
+              make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
       }
-      const float* arow = p.A + (tc.a_row + local) * p.K;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c = h ? c1 : c0;
-#pragma unroll
-        for (int j = 0; j < NC / 2; ++j) {
-          float& v = acc[h * (NC / 2) + j];
-          if (!finite(v)) {
-            const int col = GLU && h ? c + j - BN / 2 : c + j;
-            if (col < n_left) v = fma_dot(arow, (GLU && h ? p.B2 : p.B) + (tc.b_row + col) * p.K, p.K);
+      asm volatile("bar.sync 1, %0;" ::"r"(NUM_THREADS) : "memory");
+      constexpr int V = BN_OUT / 4;  // float4 per row of the output tile
+#pragma unroll 1
+      for (int i = threadIdx.x; i < BM * V; i += NUM_THREADS) {
+        const int local = i / V, c = i % V * 4;
+        if (!ok || local >= m_left || c >= n_left) continue;  // N is a multiple of 8
+        const long long out_row = p.out_row_base + row0[tc.g] + (long long)tc.m_blk * BM + local;
+        long long dest = out_row;
+        float sc = 1.0f;
+        if (EPI == EPI_SCATTER) {
+          dest = p.perm ? p.perm[out_row] : out_row;
+          if (dest < 0 || dest >= p.row_limit) {
+            atomicOr(&g_f32_error, 2u);
+            continue;
           }
+          if (p.scale) sc = p.scale[dest];
+        }
+        float v[4], w[4];
+        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(tile_out + local * C::PITCH + c);
+        if (GLU) *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(tile_out + local * C::PITCH + BN / 2 + c);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float* arow = p.A + (tc.a_row + local) * p.K;
+          const long long brow = (tc.b_row + c + u) * p.K;
+          if (!finite(v[u])) v[u] = fma_dot(arow, p.B + brow, p.K);
+          if (EPI == EPI_GELU) v[u] = gelu_erf(v[u]);
+          if (GLU) {
+            if (!finite(w[u])) w[u] = fma_dot(arow, p.B2 + brow, p.K);
+            v[u] = silu(v[u]) * w[u];
+          }
+          if (EPI == EPI_SCATTER) v[u] *= sc;
+        }
+        const float4 o = make_float4(v[0], v[1], v[2], v[3]);
+        const long long col = (long long)tc.n_blk * BN_OUT + c;
+        if (EPI == EPI_REPLICATE) {
+          for (int r = 0; r < p.rep_k; ++r)
+            *reinterpret_cast<float4*>(p.out + (long long)p.perm[out_row * p.rep_k + r] * p.ldo + col) = o;
+          if (p.self_row_base >= 0) *reinterpret_cast<float4*>(p.out + (p.self_row_base + out_row) * p.ldo + col) = o;
+        } else {
+          *reinterpret_cast<float4*>(p.out + dest * p.ldo + col) = o;
         }
       }
-      constexpr int RUNS = GLU ? 1 : 2;
-#pragma unroll
-      for (int h = 0; h < RUNS; ++h) {
-        const int c = h ? c1 : c0;
-#pragma unroll
-        for (int j = 0; j < NC / 2; j += 4) {
-          if (c + j >= n_left) continue;  // N is a multiple of 8
-          float v[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            v[u] = acc[h * (NC / 2) + j + u];
-            if (EPI == EPI_GELU) v[u] = gelu_erf(v[u]);
-            if (GLU) v[u] = silu(v[u]) * acc[NC / 2 + j + u];
-            if (EPI == EPI_SCATTER) v[u] *= sc;
-          }
-          const float4 o = make_float4(v[0], v[1], v[2], v[3]);
-          const long long col = (long long)tc.n_blk * BN_OUT + c + j;
-          if (EPI == EPI_REPLICATE) {
-            for (int r = 0; r < p.rep_k; ++r)
-              *reinterpret_cast<float4*>(p.out + (long long)p.perm[out_row * p.rep_k + r] * p.ldo + col) = o;
-            if (p.self_row_base >= 0)
-              *reinterpret_cast<float4*>(p.out + (p.self_row_base + out_row) * p.ldo + col) = o;
-          } else {
-            *reinterpret_cast<float4*>(p.out + dest * p.ldo + col) = o;
-          }
-        }
-      }
+      // the tile is read before the next one's blocks overwrite it
+      asm volatile("bar.sync 1, %0;" ::"r"(NUM_THREADS) : "memory");
     }
     if (threadIdx.x == 0 && any && (!ok || *abort_flag)) {
       // All MMAs issued so far must finish before TMEM is freed.
