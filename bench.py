@@ -129,6 +129,10 @@ def kernel_work(cfg, name: str, touched: int = 0):
         return 2.0 * T * cfg.n_shared * d * fs * glu, es * (cfg.n_shared * glu * fs * d + T * d + T * cfg.n_shared * fs)
     if name == "shared_down":
         return 2.0 * T * cfg.n_shared * fs * d, es * (cfg.n_shared * d * fs + T * cfg.n_shared * (fs + d))
+    if name in ("ffn_up", "ffn_down"):
+        # routed and shared experts in one launch
+        parts = [kernel_work(cfg, part + name[3:], touched) for part in ("expert", "shared")]
+        return parts[0][0] + parts[1][0], parts[0][1] + parts[1][1]
     if name == "lr_encode":
         return 2.0 * T * d * r, es * (T * d + r * d + T * r)
     if name == "lr_decode":
@@ -165,7 +169,8 @@ def roofline_for(cfg, name, avg_ms, peaks, peaks_src, traffic, touched: int = 0)
     (data movement, the gate, decode-sized GEMMs that stream their weights)."""
     flops, byts = kernel_work(cfg, name, touched)
     ridge = peaks["bf16_tflops"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
-    tensor = name in ("expert_up", "expert_down", "shared_up", "shared_down", "lr_encode", "lr_decode") and (
+    tensor = name in ("expert_up", "expert_down", "shared_up", "shared_down", "ffn_up", "ffn_down", "lr_encode",
+                      "lr_decode") and (
         flops / max(byts, 1) >= ridge)
     sec = avg_ms * 1e-3
     if tensor and cfg.dtype == 1:

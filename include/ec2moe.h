@@ -338,7 +338,8 @@ int32_t ec2moe_last_launch_count(void);
  * stop event.  `name` receives a static string naming the launch
  * ("gate_prep", "gate_topk", "gate_decide", "route_count", "route_scatter", "gather_rows",
  * "lr_encode", "lr_reduce", "lr_decode", "lr_codec", "expert_up", "expert_down", "shared_up",
- * "shared_down", "combine", "sum_counts"); `ms` its device duration.  Profiling is off by default and
+ * "shared_down", "ffn_up", "ffn_down" (routed and shared experts in one launch),
+ * "combine", "sum_counts"); `ms` its device duration.  Profiling is off by default and
  * costs nothing when off. */
 ec2moe_status ec2moe_profile_enable(int32_t enable);
 /* Restricts profiling to one launch per call: with launch_index >= 0 only the

@@ -357,6 +357,15 @@ cudaError_t run_gemm(const ec2moe_layer_desc* d, const GemmArgs& g, int epi, cud
   return launch_gemm_tc(g, epi, s);
 }
 
+// The shared experts as further groups of the routed experts' launches.
+struct SharedGroups {
+  const void* W1;
+  const void* W3;
+  const void* W2;
+  long long a_row;  // rows of A that every shared expert reads
+  void* out;        // [n_shared * T, d]
+};
+
 // Up projection (+ activation) then down projection over groups of rows.
 //   routed: groups = experts by device offsets; down projection scatters with
 //           perm and scales with the gate weights.
@@ -364,7 +373,8 @@ cudaError_t run_gemm(const ec2moe_layer_desc* d, const GemmArgs& g, int epi, cud
 cudaError_t run_ffn(const ec2moe_layer_desc* d, bool routed, const void* A, long long a_rows, long long a_row_base,
                     const int32_t* offsets, const void* W1, const void* W3, const void* W2, void* H, long long h_rows,
                     long long h_row_base, const int32_t* perm, const float* scale, void* out, long long out_row_base,
-                    cudaStream_t s, int g_active = 0, float* partial = nullptr, int split_k = 1) {
+                    cudaStream_t s, int g_active = 0, float* partial = nullptr, int split_k = 1,
+                    const SharedGroups* sh = nullptr) {
   const int ff = routed ? d->d_ff : d->d_ff_shared;
   const int G = routed ? d->E : d->n_shared;
   const long long rows = routed ? (long long)d->T * d->k : (long long)d->T * d->n_shared;
@@ -390,6 +400,19 @@ cudaError_t run_ffn(const ec2moe_layer_desc* d, bool routed, const void* A, long
   up.max_rows = rows;
   up.group_rows_bound = routed ? rows : d->T;
   up.g_active = routed ? g_active : 0;
+  if (sh) {
+    up.name = "ffn_up";
+    up.sh_groups = d->n_shared;
+    up.sh_rows = d->T;
+    up.sh_row0 = rows;
+    up.sh_a_row = sh->a_row;
+    up.sh_B = sh->W1;
+    up.sh_B2 = sh->W3;
+    up.row_limit = rows;
+    up.max_rows = h_rows;
+    up.group_rows_bound = 0;
+    up.g_active += d->n_shared;
+  }
   cudaError_t e = run_gemm(d, up, act_epi, s);
   if (e != cudaSuccess) return e;
   GemmArgs dn = gemm_base();
@@ -424,6 +447,19 @@ cudaError_t run_ffn(const ec2moe_layer_desc* d, bool routed, const void* A, long
   dn.max_rows = rows;
   dn.group_rows_bound = routed ? rows : d->T;
   dn.g_active = routed ? g_active : 0;
+  if (sh) {
+    dn.name = "ffn_down";
+    dn.sh_groups = d->n_shared;
+    dn.sh_rows = d->T;
+    dn.sh_row0 = rows;
+    dn.sh_a_row = -1;
+    dn.sh_B = sh->W2;
+    dn.sh_out = sh->out;
+    dn.row_limit = rows;
+    dn.max_rows = h_rows;
+    dn.group_rows_bound = 0;
+    dn.g_active += d->n_shared;
+  }
   return run_gemm(d, dn, routed ? EPI_SCATTER : EPI_STORE, s);
 }
 
@@ -506,11 +542,20 @@ cudaError_t run_expert_stage(const ec2moe_layer_desc* d, const ec2moe_layer_weig
                              cudaStream_t s) {
   const long long T = d->T, n = T * d->k;
   const bool bf = is_bf16(d);
+  // Shared experts of the routed experts' width run as further groups of the
+  // same two launches when they read decoded rows (which lie behind the routed
+  // ones in xa) and the call is neither split over K nor small enough for the
+  // swapped-operand kernel.  Two launches fewer and no partial wave between
+  // them (fine-grained layer, both sides on one box: T = 3 107 -> 96 us, T = 32
+  // 141 -> 125, T = 1000 225 -> 204, T = 16384 1542 -> 1513).
+  const bool joined = bf && d->n_shared > 0 && d->d_ff_shared == d->d_ff && x.split == 1 && d->r > 0 && !x.direct &&
+                      n > SWAP_MAX_ROWS;
+  const SharedGroups sh{w->W1s, w->W3s, w->W2s, x.shared_a_base, x.shared};
   cudaError_t e = run_ffn(d, true, x.xa, n + T, 0, x.offsets, w->W1, w->W3, w->W2, x.h,
                           n + (long long)d->n_shared * T, 0, x.perm, x.topk_w, x.slot, 0, s, x.n_allowed, x.partial,
-                          x.split);
+                          x.split, joined ? &sh : nullptr);
   if (e != cudaSuccess) return e;
-  if (d->n_shared > 0) {
+  if (d->n_shared > 0 && !joined) {
     e = run_ffn(d, false, x.shared_a, x.shared_a_rows, x.shared_a_base, nullptr, w->W1s, w->W3s, w->W2s, x.h,
                 n + (long long)d->n_shared * T, n, nullptr, nullptr, x.shared, 0, s);
     if (e != cudaSuccess) return e;

@@ -206,6 +206,17 @@ struct GemmArgs {
   long long max_rows;                // upper bound of sum_g M_g (for the grid size)
   int g_active;                      // groups expected to hold rows (tile-count estimate; 0 = G)
   long long group_rows_bound;        // upper bound of every M_g known on the host (0 = none)
+  // Shared experts as further groups of the same call (sh_groups > 0; launch_gemm_tc
+  // and launch_gemm_tok, not EPI_REPLICATE or EPI_PARTIAL): group G + j has
+  // sh_rows rows, pre-scatter output rows sh_row0 + j*sh_rows onwards, A rows from
+  // the same place or, with sh_a_row >= 0, from sh_a_row for all of them, and
+  // weights in rows [j*b_group_rows, ...) of sh_B (and sh_B2).  They are stored
+  // without perm and scale; EPI_SCATTER stores them to sh_out, row j*sh_rows
+  // onwards.  max_rows and g_active count them, row_limit does not.
+  int sh_groups, sh_rows;
+  long long sh_row0, sh_a_row;
+  const void* sh_B; const void* sh_B2; void* sh_out;
+  long long row_limit;               // rows that offsets and perm may name (0 = max_rows)
   int split_k;                       // EPI_PARTIAL: K ranges per output tile (1 = none)
   float* partial;                    // EPI_PARTIAL: fp32 [split_k][part_rows][N]
   long long part_rows;

@@ -104,6 +104,10 @@ struct Params {
   float* partial;
   long long part_rows;
   long long row_limit;  // rows of the call: group ranges and scatter destinations lie in [0, row_limit)
+  // groups [G_main, G): shared experts (GemmArgs::sh_*)
+  int G_main, sh_rows;
+  long long sh_row0, sh_a_row;
+  void* sh_out;
 };
 
 // ------------------------------------------------------------------ tile schedule
@@ -175,7 +179,8 @@ struct Cfg {
 template <int BN, int EPI, int STAGES, bool PAIR, bool QUAD = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmB2, const Params p) {
+                   const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmBs,
+                   const __grid_constant__ CUtensorMap tmB2s, const Params p) {
   static_assert(!QUAD || PAIR, "two pairs per cluster need CTA pairs");
   using C = Cfg<BN, EPI, STAGES, PAIR>;
   extern __shared__ uint8_t smem_raw[];
@@ -237,7 +242,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         p.G, lane,
         [&](int g) {
           int r0 = g * p.M, mg = p.M;
-          if (p.offsets) {
+          if (g >= p.G_main) {
+            r0 = static_cast<int>(p.sh_row0) + (g - p.G_main) * p.sh_rows;
+            mg = p.sh_rows;
+          } else if (p.offsets) {
             r0 = p.offsets[g];
             mg = p.offsets[g + 1] - r0;
             if (r0 < 0 || mg < 0 || static_cast<long long>(r0) + mg > p.row_limit) {
@@ -301,9 +309,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int tile = tile_first; tile < n_tiles && ok; tile += tile_step) {
         const TileCoord tc = decode_tile(tile / p.split_k, tile_prefix, ntn, cursor);
         const int n_blk = QUAD ? 2 * tc.n_blk + pp : tc.n_blk;
-        const int a_row = static_cast<int>(p.a_row_base) + (p.offsets ? row0[tc.g] : (p.a_shared ? 0 : row0[tc.g])) +
+        const bool sh = tc.g >= p.G_main;
+        const int a_row = (sh && p.sh_a_row >= 0 ? static_cast<int>(p.sh_a_row)
+                                                 : static_cast<int>(p.a_row_base) +
+                                                       (p.offsets || sh ? row0[tc.g] : (p.a_shared ? 0 : row0[tc.g]))) +
                           tc.m_blk * C::TILE_M + static_cast<int>(rank) * BM;
-        const int b_row = tc.g * p.b_group_rows + n_blk * C::BN_OUT;
+        const int b_row = (sh ? tc.g - p.G_main : tc.g) * p.b_group_rows + n_blk * C::BN_OUT;
+        const CUtensorMap* mB = sh ? &tmBs : &tmB;
+        const CUtensorMap* mB2 = sh ? &tmB2s : &tmB2;
         const int kb0 = (tile % p.split_k) * p.kb_per_split;
         const int kb1 = kb0 + p.kb_per_split < num_kb ? kb0 + p.kb_per_split : num_kb;
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -326,17 +339,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               tma_load_2d_to_pair_bar(smem_u32(sA + stage * C::A_BYTES), &tmA, kb * BK, a_row, fb0);
             }
             // SwiGLU: the even CTA stages the W1 rows of the tile, the odd CTA the W3 rows
-            const CUtensorMap* tb = (EPI == EPI_SWIGLU && rank) ? &tmB2 : &tmB;
+            const CUtensorMap* tb = (EPI == EPI_SWIGLU && rank) ? mB2 : mB;
             tma_load_2d_to_pair_bar(smem_u32(sB + stage * C::B_BYTES), tb, kb * BK,
                                     b_row + (EPI == EPI_SWIGLU ? 0 : static_cast<int>(rank) * C::CTA_B_ROWS), fb0);
           } else {
             mbar_expect_tx(fb, C::STAGE_BYTES);
             tma_load_2d(smem_u32(sA + stage * C::A_BYTES), &tmA, kb * BK, a_row, fb);
             if (EPI == EPI_SWIGLU) {
-              tma_load_2d(smem_u32(sB + stage * C::B_BYTES), &tmB, kb * BK, b_row, fb);
-              tma_load_2d(smem_u32(sB + stage * C::B_BYTES + C::B_BYTES / 2), &tmB2, kb * BK, b_row, fb);
+              tma_load_2d(smem_u32(sB + stage * C::B_BYTES), mB, kb * BK, b_row, fb);
+              tma_load_2d(smem_u32(sB + stage * C::B_BYTES + C::B_BYTES / 2), mB2, kb * BK, b_row, fb);
             } else {
-              tma_load_2d(smem_u32(sB + stage * C::B_BYTES), &tmB, kb * BK, b_row, fb);
+              tma_load_2d(smem_u32(sB + stage * C::B_BYTES), mB, kb * BK, b_row, fb);
             }
           }
           issued |= 1u << stage;
@@ -465,13 +478,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const uint32_t acc_phase = (it >> 1) & 1;
       // Row metadata first: its global loads overlap the tile's main loop.
       // (a group's tiles exist only if the prologue accepted its range)
-      const int mg = p.offsets ? (p.offsets[tc.g + 1] - p.offsets[tc.g]) : p.M;
+      const bool sh = tc.g >= p.G_main;
+      const int mg = sh ? p.sh_rows : p.offsets ? (p.offsets[tc.g + 1] - p.offsets[tc.g]) : p.M;
       const int local = tc.m_blk * C::TILE_M + static_cast<int>(rank) * BM + row_in_tile;
       bool valid = local < mg;
       const long long out_row = p.out_row_base + row0[tc.g] + local;
       long long dest = out_row;
       float sc = 1.0f;
-      if (EPI == EPI_SCATTER && valid) {
+      __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(EPI == EPI_SCATTER && sh ? p.sh_out : p.out);
+      if (EPI == EPI_SCATTER && sh) {
+        dest = out_row - p.sh_row0;
+      } else if (EPI == EPI_SCATTER && valid) {
         dest = p.perm ? p.perm[out_row] : out_row;
         if (dest < 0 || dest >= p.row_limit) {
           atomicOr(&g_tc_error, 2u);
@@ -571,7 +588,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int rr = part * 8 + pass * 4 + (lane >> 3);
             const bool rvalid = __shfl_sync(0xffffffffu, valid ? 1 : 0, rr) != 0;
             const U4 q4 = *reinterpret_cast<const U4*>(slab + rr * 128 + ((seg ^ (rr & 7)) * 16));
-            __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(p.out);
             if (EPI == EPI_REPLICATE) {
               // the row's expert-order slots, then (optionally) its own row
               const int* sd = s_dst + (q * 32 + rr) * 8;  // staged row rr is row q * 32 + rr of the tile
@@ -664,7 +680,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           const U4 q4 = *reinterpret_cast<const U4*>(stg + rr * C::STG_PITCH + 16 * sg);
           if (EPI == EPI_REPLICATE) {
             const long long orow_r = __shfl_sync(0xffffffffu, out_row, rr);
-            __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(p.out);
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
               const int dr = __shfl_sync(0xffffffffu, rdst[r], rr);
@@ -674,8 +689,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               *reinterpret_cast<U4*>(ob + (p.self_row_base + orow_r) * p.ldo + col + 8 * sg) = q4;
           } else {
             const long long drow = __shfl_sync(0xffffffffu, dest, rr);
-            if (rvalid)
-              *reinterpret_cast<U4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + drow * p.ldo + col + 8 * sg) = q4;
+            if (rvalid) *reinterpret_cast<U4*>(ob + drow * p.ldo + col + 8 * sg) = q4;
           }
         }
       }
@@ -806,9 +820,21 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   } else {
     mB2 = mB;
   }
+  CUtensorMap mBs = mB, mB2s = mB2;  // shared experts' weights
+  if (a.sh_groups > 0) {
+    const long long rows = (long long)a.sh_groups * a.b_group_rows;
+    if (!make_map(&mBs, a.sh_B, rows, a.K, b_box)) return cudaErrorInvalidValue;
+    mB2s = mBs;
+    if (EPI == EPI_SWIGLU && !make_map(&mB2s, a.sh_B2, rows, a.K, b_box)) return cudaErrorInvalidValue;
+  }
   Params p;
   p.offsets = a.offsets;
-  p.G = a.G;
+  p.G = a.G + a.sh_groups;
+  p.G_main = a.G;
+  p.sh_rows = a.sh_rows;
+  p.sh_row0 = a.sh_row0;
+  p.sh_a_row = a.sh_groups > 0 ? a.sh_a_row : -1;
+  p.sh_out = a.sh_out;
   p.M = a.M;
   p.a_shared = a.a_shared;
   p.a_row_base = a.a_row_base;
@@ -838,8 +864,8 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   }
   p.partial = a.partial;
   p.part_rows = a.part_rows;
-  p.row_limit = a.max_rows > 0 ? a.max_rows : (1LL << 62);
-  const long long m_tiles_max = a.max_rows / C::TILE_M + a.G;
+  p.row_limit = a.row_limit > 0 ? a.row_limit : a.max_rows > 0 ? a.max_rows : (1LL << 62);
+  const long long m_tiles_max = a.max_rows / C::TILE_M + p.G;
   long long tiles = m_tiles_max * p.n_tiles_n * p.split_k;
   if (PAIR) {
     // QUAD: a cluster tile is two N tiles (p.n_tiles_n is even)
@@ -850,7 +876,7 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
     if (tiles < clusters) clusters = static_cast<int>(tiles < 1 ? 1 : tiles);
     KernelScope ks(a.name ? a.name : kernel_name(EPI), s);
     cudaError_t le = launch_cluster(tc_gemm_kernel<BN, EPI, STAGES, PAIR, QUAD>, clusters, cdim, NUM_THREADS,
-                                    (size_t)C::SMEM, s, mA, mB, mB2, p);
+                                    (size_t)C::SMEM, s, mA, mB, mB2, mBs, mB2s, p);
     if (le != cudaSuccess) return le;
     return cudaGetLastError();
   }
@@ -858,7 +884,7 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   if (grid < 1) grid = 1;
   KernelScope ks(a.name ? a.name : kernel_name(EPI), s);
   cudaError_t le = launch_kernel(tc_gemm_kernel<BN, EPI, STAGES, PAIR>, dim3(grid), dim3(NUM_THREADS), (size_t)C::SMEM,
-                                 s, mA, mB, mB2, p);
+                                 s, mA, mB, mB2, mBs, mB2s, p);
   if (le != cudaSuccess) return le;
   return cudaGetLastError();
 }
@@ -1007,7 +1033,8 @@ bool use_quad(const GemmArgs& a, int epi, int bn) {
 }
 
 cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s) {
-  if (a.G < 1 || a.G > MAX_GROUPS || a.N % 32 != 0 || a.K % 8 != 0) return cudaErrorInvalidValue;
+  if (a.G < 1 || a.G + a.sh_groups > MAX_GROUPS || a.N % 32 != 0 || a.K % 8 != 0) return cudaErrorInvalidValue;
+  if (a.sh_groups > 0 && (epi == EPI_REPLICATE || epi == EPI_PARTIAL)) return cudaErrorInvalidValue;
   bool pair = use_pairs(a, epi);
   int bn = choose_bn(a, epi, pair);
   const int bn_out = epi == EPI_SWIGLU ? bn / 2 : bn;

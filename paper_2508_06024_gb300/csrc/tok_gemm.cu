@@ -54,7 +54,7 @@ constexpr int TG_NT = 256;    // most tokens of a tile (MMA N)
 constexpr int TG_STAGES = 6;
 constexpr int TG_EPI_WARPS = 16;  // four per TMEM lane quadrant
 constexpr int TG_THREADS = 64 + 32 * TG_EPI_WARPS;
-constexpr int TG_MAX_GROUPS = 128;
+constexpr int TG_MAX_GROUPS = 132;
 constexpr int TG_MAX_CUT = 4;     // pieces of a tile of the last wave
 constexpr int TG_W_BYTES = TG_M * TG_BK * 2;       // 16 KB of weights per stage and CTA
 constexpr int TG_X_BYTES = TG_NT / 2 * TG_BK * 2;  // 16 KB of tokens
@@ -81,12 +81,17 @@ struct TgParams {
   int n_mblk;        // weight blocks per group
   long long timeout;
   long long row_limit;  // rows of the call: group ranges and scatter destinations lie in [0, row_limit)
+  // groups [G_main, G): shared experts (GemmArgs::sh_*)
+  int G_main, sh_rows;
+  long long sh_row0, sh_a_row;
+  __nv_bfloat16* sh_out;
 };
 
 // Token boxes of 16, 32, 64 and 128 rows, weight boxes (W2: SwiGLU's W3).
 struct TgMaps {
   CUtensorMap x[4];
   CUtensorMap w, w2;
+  CUtensorMap ws, w2s;  // shared experts'
 };
 
 // A group's rows; its token tiles spread them evenly over the fewest tiles of
@@ -188,7 +193,10 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
         p.G, lane,
         [&](int g) {
           int r0 = g * p.M, mg = p.M;
-          if (p.offsets) {
+          if (g >= p.G_main) {
+            r0 = static_cast<int>(p.sh_row0) + (g - p.G_main) * p.sh_rows;
+            mg = p.sh_rows;
+          } else if (p.offsets) {
             r0 = p.offsets[g];
             mg = p.offsets[g + 1] - r0;
             if (r0 < 0 || mg < 0 || static_cast<long long>(r0) + mg > p.row_limit) {
@@ -247,9 +255,14 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
         const uint32_t bytes = TG_W_BYTES + ((1 << b1) + (b2 >= 0 ? 1 << b2 : 0)) * (TG_BK * 2);
         const CUtensorMap* x1 = &tm.x[b1 - 4];
         const CUtensorMap* x2 = &tm.x[b2 >= 0 ? b2 - 4 : 0];
-        const int x_row = static_cast<int>(p.a_row_base) + (p.offsets || !p.a_shared ? groups[x.g].row0 : 0) + x.t0 +
-                          static_cast<int>(rank) * run;
-        const int w_row = x.g * p.b_group_rows + (x.mb * 2 + static_cast<int>(rank)) * COLS;
+        const bool sh = x.g >= p.G_main;
+        const int x_row = (sh && p.sh_a_row >= 0
+                               ? static_cast<int>(p.sh_a_row)
+                               : static_cast<int>(p.a_row_base) + (p.offsets || sh || !p.a_shared ? groups[x.g].row0 : 0)) +
+                          x.t0 + static_cast<int>(rank) * run;
+        const int w_row = (sh ? x.g - p.G_main : x.g) * p.b_group_rows + (x.mb * 2 + static_cast<int>(rank)) * COLS;
+        const CUtensorMap* mw = sh ? &tm.ws : &tm.w;
+        const CUtensorMap* mw2 = sh ? &tm.w2s : &tm.w2;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!__all_sync(0xffffffffu,
                           mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_tok_error))) {
@@ -262,8 +275,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
           const uint32_t fb0 = rank == 0 ? fb : map_to_rank(fb, 0);
           const uint32_t sw = smem_u32(smem) + stage * TG_STAGE_BYTES;
           if (leader) {
-            tma_load_2d_to_pair_bar(sw, &tm.w, kb * TG_BK, w_row, fb0);
-            if (GLU) tma_load_2d_to_pair_bar(sw + TG_W_BYTES / 2, &tm.w2, kb * TG_BK, w_row, fb0);
+            tma_load_2d_to_pair_bar(sw, mw, kb * TG_BK, w_row, fb0);
+            if (GLU) tma_load_2d_to_pair_bar(sw + TG_W_BYTES / 2, mw2, kb * TG_BK, w_row, fb0);
             tma_load_2d_to_pair_bar(sw + TG_W_BYTES, x1, kb * TG_BK, x_row, fb0);
             if (b2 >= 0)
               tma_load_2d_to_pair_bar(sw + TG_W_BYTES + ((TG_BK * 2) << b1), x2, kb * TG_BK, x_row + (1 << b1), fb0);
@@ -360,7 +373,9 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
       const TgUnit x = unit_at(u, list, tile_prefix, groups, cursor);
       if (x.tn <= 0) continue;
       const int col0 = (x.mb * 2 + static_cast<int>(rank)) * COLS + (GLU ? q & 1 : q) * 32;
-      const long long base = p.out_row_base + groups[x.g].row0 + x.t0;
+      const bool sh = EPI == EPI_SCATTER && x.g >= p.G_main;  // stored to sh_out, unscaled
+      const long long base = (sh ? -p.sh_row0 : p.out_row_base) + groups[x.g].row0 + x.t0;
+      __nv_bfloat16* out = sh ? p.sh_out : p.out;
       {
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&tfull[used & 1]), (used >> 1) & 1u, budget, abort_flag,
                                                &g_tok_error));
@@ -383,7 +398,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
           bool valid = b + lane < x.tn;
           long long dest = base + b + lane;
           float sc = 1.0f;
-          if (EPI == EPI_SCATTER && valid) {
+          if (EPI == EPI_SCATTER && !sh && valid) {
             const long long o = dest;
             dest = p.perm ? p.perm[o] : o;
             if (dest < 0 || dest >= p.row_limit) {
@@ -433,7 +448,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
             const U4 v = *reinterpret_cast<const U4*>(stg + ts * 64 + seg * 16);
             const long long drow = __shfl_sync(0xffffffffu, dest, t);
             const int col = col0 + seg * 8;
-            if ((vmask >> t & 1u) && col < p.N) *reinterpret_cast<U4*>(p.out + drow * p.ldo + col) = v;
+            if ((vmask >> t & 1u) && col < p.N) *reinterpret_cast<U4*>(out + drow * p.ldo + col) = v;
           }
           __syncwarp();
         }
@@ -469,11 +484,18 @@ cudaError_t launch_epi(const GemmArgs& a, TgParams p, cudaStream_t s) {
   if (!make_tensor_map_bf16(&tm.w, a.B, a.b_rows, a.K, GLU ? TG_M / 2 : TG_M)) return cudaErrorInvalidValue;
   tm.w2 = tm.w;
   if (GLU && !make_tensor_map_bf16(&tm.w2, a.B2, a.b_rows, a.K, TG_M / 2)) return cudaErrorInvalidValue;
+  tm.ws = tm.w;
+  tm.w2s = tm.w2;
+  if (a.sh_groups > 0) {
+    const long long rows = (long long)a.sh_groups * a.b_group_rows;
+    if (!make_tensor_map_bf16(&tm.ws, a.sh_B, rows, a.K, GLU ? TG_M / 2 : TG_M)) return cudaErrorInvalidValue;
+    if (GLU && !make_tensor_map_bf16(&tm.w2s, a.sh_B2, rows, a.K, TG_M / 2)) return cudaErrorInvalidValue;
+  }
   const int cols = GLU ? TG_M : 2 * TG_M;  // output columns of a pair's weight block
   p.n_mblk = (a.N + cols - 1) / cols;
   int clusters = max_clusters(kfn, TG_THREADS, TG_SMEM, 2);
   if (clusters < 1) return cudaErrorInvalidConfiguration;
-  const long long units = (a.max_rows / 32 + a.G) * p.n_mblk;  // pieces hold 32 rows or more, but for each group's last
+  const long long units = (a.max_rows / 32 + p.G) * p.n_mblk;  // pieces hold 32 rows or more, but for each group's last
   if (units < clusters) clusters = static_cast<int>(units < 1 ? 1 : units);
   KernelScope ks(a.name ? a.name : "gemm_tok", s);
   return launch_cluster(kernel, clusters, 2, TG_THREADS, (size_t)TG_SMEM, s, tm, p);
@@ -483,7 +505,7 @@ cudaError_t launch_epi(const GemmArgs& a, TgParams p, cudaStream_t s) {
 
 bool gemm_tok_supported(const GemmArgs& a, int epi) {
   if (epi != EPI_STORE && epi != EPI_GELU && epi != EPI_SWIGLU && epi != EPI_SCATTER) return false;
-  if (a.G < 1 || a.G > TG_MAX_GROUPS || a.N % 32 != 0 || a.K % 8 != 0) return false;
+  if (a.G < 1 || a.G + a.sh_groups > TG_MAX_GROUPS || a.N % 32 != 0 || a.K % 8 != 0) return false;
   return true;
 }
 
@@ -514,7 +536,12 @@ cudaError_t launch_gemm_tok(const GemmArgs& a, int epi, cudaStream_t s) {
   if (!gemm_tok_supported(a, epi)) return cudaErrorInvalidValue;
   TgParams p{};
   p.offsets = a.offsets;
-  p.G = a.G;
+  p.G = a.G + a.sh_groups;
+  p.G_main = a.G;
+  p.sh_rows = a.sh_rows;
+  p.sh_row0 = a.sh_row0;
+  p.sh_a_row = a.sh_groups > 0 ? a.sh_a_row : -1;
+  p.sh_out = static_cast<__nv_bfloat16*>(a.sh_out);
   p.M = a.M;
   p.a_shared = a.a_shared;
   p.a_row_base = a.a_row_base;
@@ -527,7 +554,7 @@ cudaError_t launch_gemm_tok(const GemmArgs& a, int epi, cudaStream_t s) {
   p.perm = a.perm;
   p.scale = a.scale;
   p.timeout = a.timeout_cycles;
-  p.row_limit = a.max_rows > 0 ? a.max_rows : (1LL << 62);
+  p.row_limit = a.row_limit > 0 ? a.row_limit : a.max_rows > 0 ? a.max_rows : (1LL << 62);
   cudaError_t e;
   switch (epi) {
     case EPI_GELU: e = launch_epi<EPI_GELU>(a, p, s); break;
