@@ -17,22 +17,25 @@
 // FMA sums of a CUDA-core kernel: relative error of a layer's Y 5.1e-7
 // against 1.3e-6 (d = 768, d_ff = 3072), 4.4e-7 against 8.7e-7 (512, 1024).
 //
-// What bounds it: per 64-column block the 24 MMAs (M = 128, N = 128, K = 16)
-// read 192 KB of shared memory and the split writes 96 KB, 2250 clocks at 128
-// bytes per clock, beside ~1600 clocks of issue for the split, the loads and
-// the drain; a timing copy without the MMAs still takes 3/4 of the time, one
-// without the global loads all of it.  Measured (expert_up / expert_down of 12
-// experts, 1024 rows, 768 x 3072): CUDA-core tiles 426 / 758 us, here 70 / 65.
+// What bounds it: a chain of nearly equal parts per 64-column block.  A pass of
+// a layer (12 experts, 1024 rows, 768 x 3072; the two expert GEMMs are 4/5 of
+// it) takes 155 us, copies of the kernel without the MMAs 128, with half of
+// them 133, without B's split and stores 142, without the loads 142, without
+// A's stores 150.  With A's terms in shared memory as well, where the MMAs then
+// read twice as much, it takes 162.  CUDA-core tiles took 426 us for expert_up
+// alone and 758 for expert_down.
 //
 // One persistent CTA of 16 warps per SM (a 17th warp for the MMAs alone would
-// cut the registers per thread from 128 to 96).  Every warp loads A and B
-// blocks as fp32 (16 bytes per lane, whole 256-byte row pieces, one block
-// ahead in registers), writes the three terms into the swizzled K-major stage,
-// and drains the previous segment's accumulators (warp w reads TMEM lanes 32
-// (w % 4) .. +31 and a quarter of the columns); at the end of the tile it
-// applies the epilogue from registers.  Thread 0 also issues the MMAs.
-// Two stages and two pairs of accumulators, so a block is loaded and split
-// while the previous one multiplies.  Every wait is bounded; a timeout sets
+// cut the registers per thread from 128 to 96).  Every warp loads A and B blocks
+// as fp32, one block ahead in registers, and writes the three terms: of A into
+// tensor memory (a thread's row is its TMEM lane; a warp takes a quarter of the
+// block's columns), of B into the swizzled K-major stage (16 bytes per lane,
+// whole 256-byte row pieces).  It drains the finished segment's accumulators
+// (TMEM lanes 32 (w % 4) .. +31, a quarter of the columns) and at the end of the
+// tile applies the epilogue.  Warp 0 also issues the MMAs.
+// Two stages, so a block is loaded and split while the previous one multiplies;
+// two pairs of accumulators for 64-wide tiles, one for 128-wide ones (the A
+// stages take the other pair's columns).  Every wait is bounded; a timeout sets
 // the error word and the CTA ends after its MMAs in flight.
 //
 // A result that is not finite (an infinite or NaN operand, an operand that
@@ -80,6 +83,7 @@ struct FParams {
   int n_tiles_n;
   int split;          // CTAs of a cluster sharing a tile's K range (1: no cluster)
   int kb_per_split;
+  int wide_a;         // A is 32-byte aligned: 256-bit loads
   long long a_rows;
   long long timeout;
   long long row_limit;  // rows of the call: group ranges and scatter destinations lie in [0, row_limit)
@@ -87,24 +91,29 @@ struct FParams {
 
 template <int BN>
 struct FCfg {
-  static constexpr int A_BYTES = BM * BK * 2;  // one term of the A block
-  static constexpr int B_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = 3 * (A_BYTES + B_BYTES);
-  static constexpr int OFF_BARS = STAGES * STAGE_BYTES;
+  static constexpr int B_BYTES = BN * BK * 2;  // one term of the B block
+  static constexpr int STAGE_BYTES = 3 * B_BYTES;
+  static constexpr int NC = BN / 4;            // accumulator columns of a thread
+  static constexpr int PITCH = BN + 4;         // floats per row of the result tile (conflict-free 16-byte columns)
+  // the stages; the other CTAs' sums and the result tile use the space between tiles
+  static constexpr int SUM_BYTES = (MAX_SPLIT - 1) * NUM_THREADS * NC * 4;
+  static constexpr int DATA_BYTES = (SUM_BYTES > 120 * 1024 ? SUM_BYTES : 120 * 1024);  // one CTA per SM in any case
+  static constexpr int OFF_BARS = DATA_BYTES;
   static constexpr int N_BARS = 2 * STAGES + 5;
   static constexpr int OFF_SLOT = OFF_BARS + N_BARS * 8;  // TMEM address, abort flag
   static constexpr int OFF_PREFIX = OFF_SLOT + 16;
   static constexpr int OFF_ROW0 = OFF_PREFIX + (MAX_GROUPS + 1) * 4;
   static constexpr int SMEM = 1024 + OFF_ROW0 + MAX_GROUPS * 4;
-  static constexpr int TMEM_COLS = 4 * BN;  // two pairs of accumulators
-  static constexpr int NC = BN / 4;         // accumulator columns of a thread
-  static constexpr int PITCH = BN + 4;      // floats per row of the result tile (conflict-free 16-byte columns)
-  static constexpr int A_CHUNKS = BM * BK / 4 / NUM_THREADS;  // 16-byte pieces per thread and block
-  static constexpr int B_CHUNKS = BN * BK / 4 / NUM_THREADS;
+  // Tensor memory: N_ACC pairs of accumulators, then two stages of A terms (a
+  // term is 32 columns: 64 bf16 per lane, two to a column).
+  static constexpr int N_ACC = BN == 64 ? 2 : 1;
+  static constexpr int A_COL = N_ACC * 2 * BN;
+  static constexpr int A_TERM = BK / 2;
+  static constexpr int TMEM_COLS = 512;
+  static constexpr int B_CHUNKS = BN * BK / 4 / NUM_THREADS;  // 16-byte pieces of B per thread and block
+  static_assert(STAGES * STAGE_BYTES <= DATA_BYTES && A_COL + STAGES * 3 * A_TERM <= TMEM_COLS, "on-chip memory");
   static_assert(SMEM <= 232448 && OFF_BARS % 1024 == 0, "shared memory per CTA");
-  static_assert((MAX_SPLIT - 1) * NUM_THREADS * NC * 4 <= STAGES * STAGE_BYTES, "the other CTAs' sums fit the stages");
-  static_assert(BM * PITCH * 4 <= STAGES * STAGE_BYTES, "the result tile fits the stages");
-  static_assert(TMEM_COLS == 256 || TMEM_COLS == 512, "TMEM allocation");
+  static_assert(BM * PITCH * 4 <= DATA_BYTES, "the result tile fits");
 };
 
 // Packed pairs of fp32 (one instruction for two additions).
@@ -222,7 +231,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
   int* tile_prefix = reinterpret_cast<int*>(smem + C::OFF_PREFIX);
   int* row0 = reinterpret_cast<int*>(smem + C::OFF_ROW0);
   float* tile_out = reinterpret_cast<float*>(smem);  // the result tile, over the stages
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // warp-uniform for the compiler
   const int lane = threadIdx.x & 31;
   pdl_trigger();
   if (threadIdx.x == 0) {
@@ -286,7 +295,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
     // same output columns of W1 and of W3)
     const int c0 = GLU ? part * (NC / 2) : part * NC;
     const int c1 = GLU ? BN / 2 + part * (NC / 2) : part * NC + NC / 2;
-    // 16-byte pieces: rows lr + 32 i, columns lc .. lc + 3 of a block
+    // A: this thread's row is its TMEM lane, 16 columns of a block (its warp's
+    // quarter).  B: 16-byte pieces, rows lr + 32 i, columns lc .. lc + 3.
+    const int ac0 = part * 16;
+    const bool wide_a = p.wide_a != 0;
     const int lr = threadIdx.x >> 4;
     const int lc = (threadIdx.x & 15) * 4;
     const int soff = lr * 128 + (((lc >> 3) ^ (lr & 7)) << 4) + ((lc >> 2) & 1) * 8;
@@ -294,66 +306,85 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
     int it = 0;   // blocks so far: stage it & 1
     int seg = 0;  // segments so far: accumulator pair seg & 1
     bool ok = true, any = false;
-    // The MMAs of block i of segment sg, by thread 0 once every warp has written its part.
+    // The MMAs of block i of segment sg, by warp 0 once every warp has written
+    // its part.  The warp index, the stage and the accumulator go through a
+    // shuffle, which tells the compiler that they are warp-uniform, so that the
+    // operands of the 24 MMAs stay in uniform registers; one elected lane issues.
     auto multiply = [&](int i, int sg, bool first, bool last) {
       constexpr uint32_t IDESC = idesc_bf16(BM, BN);
-      constexpr uint64_t DA = C::A_BYTES >> 4, DB = C::B_BYTES >> 4;  // next term
-      const int st = i & 1, ac = sg & 1;
-      if ((first && !mbar_wait(smem_u32(&tempty[ac]), (static_cast<uint32_t>(sg >> 1) & 1u) ^ 1u, budget, abort_flag,
-                               &g_f32_error)) ||
-          !mbar_wait(smem_u32(&full[st]), static_cast<uint32_t>(i >> 1) & 1u, budget, abort_flag, &g_f32_error))
+      constexpr uint64_t DB = C::B_BYTES >> 4;  // next term of B
+      const int st = __shfl_sync(0xffffffffu, i & 1, 0), ac = __shfl_sync(0xffffffffu, sg % C::N_ACC, 0);
+      const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
+      const bool issue = elect_one();
+      if ((first && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&tempty[ac]), (static_cast<uint32_t>(sg / C::N_ACC) & 1u) ^ 1u,
+                                                       budget, abort_flag, &g_f32_error))) ||
+          !__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), static_cast<uint32_t>(i >> 1) & 1u, budget, abort_flag,
+                                             &g_f32_error)))
         return;  // the abort flag is up: every later wait of the CTA fails too
       tc_fence_after();
-      const uint64_t da = sdesc_sw128(smem_u32(smem + st * C::STAGE_BYTES));
-      const uint64_t db = sdesc_sw128(smem_u32(smem + st * C::STAGE_BYTES + 3 * C::A_BYTES));
-      const uint32_t d_main = tmem_base + static_cast<uint32_t>(ac * 2 * BN);
+      const uint32_t a0 = tb + C::A_COL + st * 3 * C::A_TERM;
+      const uint64_t db = sdesc_sw128(smem_u32(smem + st * C::STAGE_BYTES));
+      const uint32_t d_main = tb + static_cast<uint32_t>(ac * 2 * BN);
       const uint32_t d_minor = d_main + BN;
+      if (issue) {
 #pragma unroll
-      for (int kk = 0; kk < BK / UK; ++kk) {
-        const uint64_t a = da + 2 * kk, b = db + 2 * kk;
-        const uint32_t more = kk || !first ? 1u : 0u;
-        umma_bf16(d_minor, a, b + 2 * DB, IDESC, more);  // x0 w2
-        umma_bf16(d_minor, a + DA, b + DB, IDESC, 1u);   // x1 w1
-        umma_bf16(d_minor, a + 2 * DA, b, IDESC, 1u);    // x2 w0
-        umma_bf16(d_minor, a, b + DB, IDESC, 1u);        // x0 w1
-        umma_bf16(d_minor, a + DA, b, IDESC, 1u);        // x1 w0
-        umma_bf16(d_main, a, b, IDESC, more);            // x0 w0
+        for (int kk = 0; kk < BK / UK; ++kk) {
+          const uint32_t a = a0 + kk * (UK / 2);
+          const uint64_t b = db + 2 * kk;
+          const uint32_t more = kk || !first ? 1u : 0u;
+          umma_bf16_ts(d_minor, a, b + 2 * DB, IDESC, more);        // x0 w2
+          umma_bf16_ts(d_minor, a + C::A_TERM, b + DB, IDESC, 1u);  // x1 w1
+          umma_bf16_ts(d_minor, a + 2 * C::A_TERM, b, IDESC, 1u);   // x2 w0
+          umma_bf16_ts(d_minor, a, b + DB, IDESC, 1u);              // x0 w1
+          umma_bf16_ts(d_minor, a + C::A_TERM, b, IDESC, 1u);       // x1 w0
+          umma_bf16_ts(d_main, a, b, IDESC, more);                  // x0 w0
+        }
+        umma_commit(smem_u32(&empty[st]));
+        if (last) umma_commit(smem_u32(&tfull[ac]));
       }
       any = true;
-      umma_commit(smem_u32(&empty[st]));
-      if (last) umma_commit(smem_u32(&tfull[ac]));
     };
     const int kb_lo = rank * p.kb_per_split;
     const int kb_hi = kb_lo + p.kb_per_split < num_kb ? kb_lo + p.kb_per_split : num_kb;
     for (int tile = tile_first; tile < n_tiles; tile += tile_step) {
       const FTile tc = tile_at(p, tile, tile_prefix, row0, cursor, BN_OUT);
       const int m_left = tc.m_left, n_left = tc.n_left;
-      // Pieces of rows that are never stored are neither split nor written;
-      // their loads read the tile's first row instead.
-      uint32_t live = 0;  // bit i: A piece i, bit 8 + i: B piece i
-      const float* src_a[C::A_CHUNKS];
+      // Rows that are never stored read the tile's first row instead; of B they
+      // are neither split nor written.
+      const int arow_l = q * 32 + lane;
+      const float* src_a =
+          p.A + (tc.a_row + (arow_l < m_left && tc.a_row + arow_l < p.a_rows ? arow_l : 0)) * p.K + ac0;
+      uint32_t live = 0;  // bit i: B piece i
       const float* src_b[C::B_CHUNKS];
-#pragma unroll
-      for (int i = 0; i < C::A_CHUNKS; ++i) {
-        const bool in = lr + 32 * i < m_left && tc.a_row + lr + 32 * i < p.a_rows;
-        live |= in ? 1u << i : 0u;
-        src_a[i] = p.A + (tc.a_row + (in ? lr + 32 * i : 0)) * p.K + lc;
-      }
 #pragma unroll
       for (int i = 0; i < C::B_CHUNKS; ++i) {
         // rows 0 .. BN_OUT - 1 of the block from B, the rest (SwiGLU) from B2
         const int r = (lr + 32 * i) % BN_OUT;
         const bool in = r < n_left;
-        live |= in ? 256u << i : 0u;
+        live |= in ? 1u << i : 0u;
         src_b[i] = (GLU && 32 * i >= BN_OUT ? p.B2 : p.B) + (tc.b_row + (in ? r : 0)) * p.K + lc;
       }
-      float4 ra[C::A_CHUNKS], rb[C::B_CHUNKS];
+      float ra[16];
+      float4 rb[C::B_CHUNKS];
       const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       auto load_a = [&](int kb) {
-        const bool in_k = kb * BK + lc < p.K;  // K is a multiple of 8: a piece is inside or outside
 #pragma unroll
-        for (int i = 0; i < C::A_CHUNKS; ++i)
-          ra[i] = in_k ? __ldg(reinterpret_cast<const float4*>(src_a[i] + kb * BK)) : zero;
+        for (int h = 0; h < 2; ++h) {
+          const int k = kb * BK + ac0 + h * 8;  // K is a multiple of 8: eight columns are inside or outside
+          float* r = ra + h * 8;
+          if (k >= p.K) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) r[u] = 0.0f;
+          } else if (wide_a) {
+            asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+                         : "l"(src_a + kb * BK + h * 8));
+          } else {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(src_a + kb * BK + h * 8));
+            const float4 y = __ldg(reinterpret_cast<const float4*>(src_a + kb * BK + h * 8 + 4));
+            r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w; r[4] = y.x; r[5] = y.y; r[6] = y.z; r[7] = y.w;
+          }
+        }
       };
       auto load_b = [&](int kb) {
         const bool in_k = kb * BK + lc < p.K;
@@ -365,16 +396,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
 #pragma unroll
       for (int j = 0; j < NC; ++j) acc[j] = 0.0f;
       auto drain_segment = [&](int i) {  // segment i of this CTA
-        const int st = i & 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tfull[st]), static_cast<uint32_t>(i >> 1) & 1u, budget,
+        const int ac = i % C::N_ACC;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tfull[ac]), static_cast<uint32_t>(i / C::N_ACC) & 1u, budget,
                                                abort_flag, &g_f32_error)))
           return false;
         tc_fence_after();
-        const uint32_t t = t_row + static_cast<uint32_t>(st * 2 * BN);
+        const uint32_t t = t_row + static_cast<uint32_t>(ac * 2 * BN);
         drain_add<NC>(t, t + BN, c0, c1, acc);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&tempty[st]));
+        if (lane == 0) mbar_arrive(smem_u32(&tempty[ac]));
         return true;
       };
       if (ok) {
@@ -388,28 +419,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
           ok = false;
           break;
         }
-        uint8_t* sa = smem + st * C::STAGE_BYTES + soff;
-        uint8_t* sb = sa + 3 * C::A_BYTES;
+        tc_fence_after();
+        {
+          uint32_t t0[8], t1[8], t2[8];
 #pragma unroll
-        for (int i = 0; i < C::A_CHUNKS; ++i) {
-          if (!(live >> i & 1u)) continue;  // rows that are never stored
-          uint2 t0, t1, t2;
-          split3(ra[i], t0, t1, t2);
-          *reinterpret_cast<uint2*>(sa + i * 4096) = t0;
-          *reinterpret_cast<uint2*>(sa + i * 4096 + C::A_BYTES) = t1;
-          *reinterpret_cast<uint2*>(sa + i * 4096 + 2 * C::A_BYTES) = t2;
+          for (int j = 0; j < 8; ++j) split3(ra[2 * j], ra[2 * j + 1], t0[j], t1[j], t2[j]);
+          const uint32_t ta = t_row + C::A_COL + st * 3 * C::A_TERM + part * 8;
+          tmem_st8(ta, t0);
+          tmem_st8(ta + C::A_TERM, t1);
+          tmem_st8(ta + 2 * C::A_TERM, t2);
         }
+        uint8_t* sb = smem + st * C::STAGE_BYTES + soff;
 #pragma unroll
         for (int i = 0; i < C::B_CHUNKS; ++i) {
-          if (!(live >> (8 + i) & 1u)) continue;
+          if (!(live >> i & 1u)) continue;
           uint2 t0, t1, t2;
           split3(rb[i], t0, t1, t2);
           *reinterpret_cast<uint2*>(sb + i * 4096) = t0;
           *reinterpret_cast<uint2*>(sb + i * 4096 + C::B_BYTES) = t1;
           *reinterpret_cast<uint2*>(sb + i * 4096 + 2 * C::B_BYTES) = t2;
         }
-        // the tensor core reads these through the async proxy
+        // the tensor core reads the B terms through the async proxy, the A terms
+        // once the stores to tensor memory have completed
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tmem_wait_st();
+        tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&full[st]));
         if (kb + 1 < kb_hi) {
@@ -418,10 +452,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
         }
         const bool first = (kb - kb_lo) % SEG == 0;
         const bool last = (kb - kb_lo) % SEG == SEG - 1 || kb + 1 == kb_hi;
-        if (threadIdx.x == 0) multiply(it, seg, first, last);
+        // The segment before this one is drained while this one multiplies, or,
+        // with one pair of accumulators, before it may.
+        if (C::N_ACC == 1 && first && kb > kb_lo && !drain_segment(seg - 1)) ok = false;
+        if (warp == 0 && ok) multiply(it, seg, first, last);
         __syncwarp();
-        // the segment before this one, while this one multiplies
-        if (first && kb > kb_lo && !drain_segment(seg - 1)) ok = false;
+        if (C::N_ACC == 2 && first && kb > kb_lo && !drain_segment(seg - 1)) ok = false;
         if (last) ++seg;
       }
       if (ok && !drain_segment(seg - 1)) ok = false;
@@ -511,7 +547,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
       // the tile is read before the next one's blocks overwrite it
       asm volatile("bar.sync 1, %0;" ::"r"(NUM_THREADS) : "memory");
     }
-    if (threadIdx.x == 0 && any && (!ok || *abort_flag)) {
+    if (warp == 0 && any && __any_sync(0xffffffffu, !ok || *abort_flag) && elect_one()) {
       // All MMAs issued so far must finish before TMEM is freed.
       umma_commit(smem_u32(drain));
       mbar_drain(smem_u32(drain), 0, DRAIN_CYCLES);
@@ -621,6 +657,7 @@ cudaError_t launch_gemm_f32(const GemmArgs& a, int epi, cudaStream_t s) {
   p.n_tiles_n = p.split = p.kb_per_split = 0;  // launch_epi
   p.a_rows = a.a_rows;
   p.timeout = a.timeout_cycles;
+  p.wide_a = reinterpret_cast<uintptr_t>(a.A) % 32 == 0;
   p.row_limit = a.max_rows > 0 ? a.max_rows : (1LL << 62);
   cudaError_t e;
   switch (epi) {

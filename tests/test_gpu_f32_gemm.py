@@ -51,6 +51,17 @@ def test_codec_f32_edges(T, d, r):
     _check(Xh, Z, Vd)
 
 
+def test_f32_rows_aligned_to_16_bytes_only():
+    T, d, r = 150, 104, 72
+    X = _randn(1, T * d + 4)[4:].view(T, d)  # 16-byte aligned, not 32
+    Ve = _randn(2, r, d)
+    desc = C.make_desc(T=T, d=d, E=8, d_ff=8, k=1, dtype=C.F32, r=r)
+    Z = torch.empty(T, r, device="cuda")
+    C.ec2moe_lr_encode(desc, X, Ve, Z)
+    assert C.ec2moe_last_device_error() == C.OK
+    _check(Z, X, Ve)
+
+
 @pytest.mark.parametrize("act", [C.GELU, C.SWIGLU], ids=["gelu", "swiglu"])
 @pytest.mark.parametrize("rows,d,ff", [([1, 0, 128, 130], 72, 40), ([0, 257, 0, 3], 200, 1096)],
                          ids=["narrow", "wide"])
