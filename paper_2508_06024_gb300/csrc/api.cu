@@ -546,7 +546,7 @@ cudaError_t run_expert_stage(const ec2moe_layer_desc* d, const ec2moe_layer_weig
   // same two launches when they read decoded rows (which lie behind the routed
   // ones in xa) and the call is neither split over K nor small enough for the
   // swapped-operand kernel.  Two launches fewer and no partial wave between
-  // them (fine-grained layer, both sides on one box: T = 3 107 -> 96 us, T = 32
+  // them (fine-grained layer, both sides on one GPU: T = 3 107 -> 96 us, T = 32
   // 141 -> 125, T = 1000 225 -> 204, T = 16384 1542 -> 1513).
   const bool joined = bf && d->n_shared > 0 && d->d_ff_shared == d->d_ff && x.split == 1 && d->r > 0 && !x.direct &&
                       n > SWAP_MAX_ROWS;

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 namespace ec2moe {
 
@@ -14,6 +15,19 @@ struct alignas(16) U4 { uint32_t x, y, z, w; };
 // complete and visible (a no-op when launched without the attribute).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// One 32-bit load under a predicate, without a branch; 0 when off.
+template <typename T>
+__device__ __forceinline__ T ld_if(bool on, const T* at) {
+  uint32_t v = 0;
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p ld.global.b32 %0, [%1];\n}"
+               : "+r"(v)
+               : "l"(at), "r"(static_cast<uint32_t>(on))
+               : "memory");
+  T out;
+  memcpy(&out, &v, sizeof(out));
+  return out;
+}
 
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }

@@ -509,7 +509,7 @@ bool gemm_tok_supported(const GemmArgs& a, int epi) {
   return true;
 }
 
-// Where this orientation is the faster one (both sides measured on one box,
+// Where this orientation is the faster one (both sides measured on one GPU,
 // us; Mixtral-shaped d = 4096, d_ff = 14336, 6 experts, and fine-grained d =
 // 2048, d_ff = 1408, 32 experts; rows per expert in brackets):
 //   up    Mixtral [85] 213 -> 219, [128] 229 -> 223, [171] 259 -> 229, [259] 298 -> 271, [512] 513 -> 450,
