@@ -829,42 +829,52 @@ __global__ void __launch_bounds__(SL_THREADS) gate_decide_kernel(const KParams p
   const int tile = pf ? 0 : blockIdx.x;
   const bool writer = !pf || blockIdx.x == 0;
   pdl_trigger();
-  pdl_wait();
   const size_t plane = (size_t)p.T * O;
-  for (int i = threadIdx.x; i < GD_SPLIT * pairs; i += SL_THREADS) {
-    const int g = i / pairs, pr = i % pairs;
-    const int tok = tile * bt + pr / O;
-    float sum = 0.0f;
-    if (tok < p.T) {
-      const float* src = part + (size_t)tok * O + pr % O;
-      for (int c0 = g; c0 < n_chunks; c0 += 8 * GD_SPLIT) {
-        float v[8];
+  // First with the loads of the previous kernel's sums predicated off and nothing
+  // written, while that kernel runs: the code comes to the SM (the weight streams
+  // of the calls before evict it from L2; fine-grained layer, T = 32: a call
+  // 125.4 -> 123.2 us).
+#pragma unroll 1
+  for (int real = 0; real < 2; ++real) {
+    if (real) pdl_wait();
+    for (int i = threadIdx.x; i < GD_SPLIT * pairs; i += SL_THREADS) {
+      const int g = i / pairs, pr = i % pairs;
+      const int tok = tile * bt + pr / O;
+      float sum = 0.0f;
+      if (tok < p.T) {
+        const float* src = part + (size_t)tok * O + pr % O;
+        const int end = real ? n_chunks : g + 1;
+#pragma unroll 1
+        for (int c0 = g; c0 < end; c0 += 8 * GD_SPLIT) {
+          float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int c = c0 + u * GD_SPLIT;
-          v[u] = c < n_chunks ? src[(size_t)c * plane] : 0.0f;
+          for (int u = 0; u < 8; ++u) {
+            const int c = c0 + u * GD_SPLIT;
+            v[u] = ld_if(real && c < n_chunks, src + (size_t)c * plane);
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) sum += v[u];  // chunk order within the group
         }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) sum += v[u];  // chunk order within the group
       }
+      sGrp[i] = sum;
     }
-    sGrp[i] = sum;
-  }
-  __syncthreads();
-  for (int pr = threadIdx.x; pr < pairs; pr += SL_THREADS) {
-    const int o = pr % O;
-    float sum = sGrp[pr];
+    __syncthreads();
+    for (int pr = threadIdx.x; pr < pairs; pr += SL_THREADS) {
+      const int o = pr % O;
+      float sum = sGrp[pr];
 #pragma unroll
-    for (int g = 1; g < GD_SPLIT; ++g) sum += sGrp[g * pairs + pr];
-    sLog[pr] = sum + (o < p.E ? p.b_local[o] : p.b_global[o - p.E]);
+      for (int g = 1; g < GD_SPLIT; ++g) sum += sGrp[g * pairs + pr];
+      sLog[pr] = sum + (o < p.E ? p.b_local[o] : p.b_global[o - p.E]);
+    }
+    __syncthreads();
+    for (int jj = warp; jj < bt; jj += SL_THREADS / 32) {
+      const int tok = tile * bt + jj;
+      if (tok < p.T)
+        decide_token_warp(p, sLog + jj * O, tok, lane, (p.route_counts || pf) ? sIdx + jj * p.k : nullptr,
+                          writer && real);
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int jj = warp; jj < bt; jj += SL_THREADS / 32) {
-    const int tok = tile * bt + jj;
-    if (tok < p.T)
-      decide_token_warp(p, sLog + jj * O, tok, lane, (p.route_counts || pf) ? sIdx + jj * p.k : nullptr, writer);
-  }
-  __syncthreads();
   if (writer && p.route_counts) route_tile(p, tile, bt, sIdx, s_base);
   if (!pf) return;
   // the chosen experts in id order (the swapped GEMM's active groups)
