@@ -70,6 +70,10 @@ constexpr int GC_MAX_O = 80;
 constexpr int GC_MAX_STAGES = 10;
 constexpr int GC_THREADS = 448;
 constexpr int GC_WORKERS = 384;     // warps 2..13
+// Without prepared rows every worker warp is busy in the main loop, so a warp of
+// its own brings the decision's code to the SM (a drain warp doing it held up
+// short main loops: fine-grained steps, T = 2001, 343 -> 340 us).
+constexpr int GC_WARM_WARP = 14;
 constexpr int GC_ACC_STRIDE = 256;  // TMEM columns between the two accumulators (3 * O_pad <= 240 each)
 constexpr int GC_CS = 2;            // CTAs per tile (cluster) when d_model is split
 constexpr int GC_SPLIT_MIN_NK = 32; // stages per tile from which d_model is split
@@ -380,7 +384,7 @@ __global__ void __launch_bounds__(256) gate_split_kernel(const float* W_local, c
 }
 
 template <int NB, bool PREP>
-__global__ void __launch_bounds__(GC_THREADS, 1)
+__global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
     gate_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                    const __grid_constant__ GcParams gp) {
   using namespace tc;
@@ -444,7 +448,7 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
     // the owned rows' partials of the other cs - 1 CTAs (one tile per cluster)
     if (cs > 1) mbar_expect_tx(smem_u32(recvb), static_cast<uint32_t>((cs - 1) * rows_own * n_pad * 4));
   }
-  for (int o = threadIdx.x - 64; o >= 0 && o < O; o += GC_THREADS - 64)
+  for (int o = threadIdx.x - 64; o >= 0 && o < O; o += PREP ? GC_THREADS - 64 : GC_THREADS - 32)
     s_bias[o] = o < p.E ? p.b_local[o] : p.b_global[o - p.E];
   if (warp == 2) {
     // the allowed experts in ascending order, and where each group's begin
@@ -593,6 +597,14 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
         mbar_drain(smem_u32(drain), 0, DRAIN_CYCLES);
       }
     }
+  } else if (!PREP && warp == GC_WARM_WARP) {
+    // the decision's code to the SM, as an idle warp does below with prepared rows
+    float* warm = reinterpret_cast<float*>(smem + L.warm_off);
+    lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
+    if (p.k == 1) pick_row<1>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+    else if (p.k == 2) pick_row<2>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+    else if (p.k <= 4) pick_row<4>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+    else pick_row<8>(p, warm, O, s_list, s_grp, 0, nullptr, false);
   } else {
     // ------------------------------------------------------------ worker warps
     const int wt = threadIdx.x - 64;
@@ -606,13 +618,27 @@ __global__ void __launch_bounds__(GC_THREADS, 1)
       else if (p.k <= 4) pick_row<4>(p, Lr, O, s_list, s_grp, tok, sx, real);
       else pick_row<8>(p, Lr, O, s_list, s_grp, tok, sx, real);
     };
-    if (warp == (PREP ? 6 : 5)) {
-      // an idle warp (without prepared rows a drain warp, which has nothing to do
-      // before the first segment ends): bring the decision's code to the SM (on a row of its own,
+    if (PREP && warp == 6) {
+      // an idle warp: bring the decision's code to the SM (on a row of its own,
       // whatever it holds; nothing reads the outcome)
       float* warm = reinterpret_cast<float*>(smem + L.warm_off);
       lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
       pick(warm, nullptr, 0, false);
+    }
+    if (!PREP && !is_drain) {
+      // The fp32 gate rows to L2: the grid's converting threads together name
+      // each 128-byte line once, so that the loads below, one stage ahead of
+      // their use, wait for L2 and not for DRAM (fine-grained steps, T = 2001:
+      // 346.5 -> 343 us; Switch-shaped, T = 665: 75.6 -> 74.3).
+      const long long row_lines = (p.d * 4LL + 127) / 128, lines = O * row_lines;
+      constexpr int conv_threads = GC_THREADS - 192;
+      for (long long i = static_cast<long long>(blockIdx.x) * conv_threads + (threadIdx.x - 192); i < lines;
+           i += static_cast<long long>(gridDim.x) * conv_threads) {
+        const int r = static_cast<int>(i / row_lines);
+        const float* src = (r < p.E ? p.W_local + (size_t)r * p.d : p.W_global + (size_t)(r - p.E) * p.d) +
+                           (i - r * row_lines) * 32;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+      }
     }
     pdl_wait();  // the routing counters are cleared by the previous kernel (PREP)
     int stage = 0;
@@ -831,11 +857,12 @@ cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(gate_tc_kernel<NB, PREP>), smem);
   if (e != cudaSuccess) return e;
   const int blocks = gc_blocks(p.T, cs);
+  const int threads = PREP ? GC_THREADS : GC_THREADS + 32;
   if (cs == 1)
-    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(GC_THREADS), (size_t)smem, s, mX, mW, gp);
+    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(threads), (size_t)smem, s, mX, mW, gp);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(GC_THREADS);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
