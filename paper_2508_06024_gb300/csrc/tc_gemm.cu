@@ -36,13 +36,6 @@
 // a cluster barrier precedes its release.  After an abort the odd CTA cannot
 // observe its own copies, so it waits a fixed, bounded time for them to land.
 //
-// Two pairs per cluster (QUAD, opt-in): four CTAs, pair p = CTAs 2p and
-// 2p + 1, both pairs on the same 256 rows of A and on N tiles 2j and 2j + 1.
-// Each CTA loads 64 of its 128 A rows and multicasts them to the CTA of the
-// same pair rank in the other pair; a destination's bytes complete on the full
-// barrier of its own pair's even CTA.  Stage-freeing commits go to all four
-// CTAs and each empty barrier counts both pairs' commits.
-//
 // Every mbarrier wait is bounded by a clock64 budget.  A wait that gives up
 // sets the device error word, raises a CTA-wide abort flag that ends every
 // other wait at once, waits (again bounded) for the CTA's own TMA copies and
@@ -176,12 +169,11 @@ struct Cfg {
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 
-template <int BN, int EPI, int STAGES, bool PAIR, bool QUAD = false>
+template <int BN, int EPI, int STAGES, bool PAIR>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmBs,
                    const __grid_constant__ CUtensorMap tmB2s, const Params p) {
-  static_assert(!QUAD || PAIR, "two pairs per cluster need CTA pairs");
   using C = Cfg<BN, EPI, STAGES, PAIR>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -203,16 +195,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  // PAIR: rank in the CTA pair (0 issues the MMAs), the pair's even CTA in
-  // the cluster, the cluster's tile stream.  QUAD: the cluster holds two pairs
-  // (CTAs 0-1 and 2-3) on the same 256 rows of A and neighbouring N tiles;
-  // each CTA loads half of its 128 A rows and multicasts them to the CTA of
-  // the same pair rank in the other pair.
-  const uint32_t crank = PAIR ? cluster_ctarank() : 0u;
-  const uint32_t rank = crank & 1u;
-  const uint32_t leader = crank & ~1u;
-  const int pp = QUAD ? static_cast<int>(crank >> 1) : 0;
-  const int ntn = QUAD ? p.n_tiles_n / 2 : p.n_tiles_n;  // N tiles of a cluster tile's stream
+  // PAIR: rank in the CTA pair (0 issues the MMAs), the pair's tile stream.
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int tile_first = PAIR ? static_cast<int>(cluster_id_x()) : static_cast<int>(blockIdx.x);
   const int tile_step = PAIR ? static_cast<int>(cluster_count_x()) : static_cast<int>(gridDim.x);
   // Barrier set-up, TMEM allocation and descriptor prefetch overlap the
@@ -222,9 +206,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
-      // QUAD: a stage is free once both pairs' MMAs have read it (the other
-      // pair multicasts into it)
-      mbar_init(smem_u32(&empty[s]), QUAD ? 2 : 1);
+      mbar_init(smem_u32(&empty[s]), 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&tfull[a]), 1);
@@ -291,7 +273,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   // Split-K (EPI_PARTIAL): tile t covers output tile t / split_k and the
   // k-blocks [ks * kb_per_split, ...) with ks = t % split_k.
-  const int n_tiles = tile_prefix[p.G] * ntn * p.split_k;
+  const int n_tiles = tile_prefix[p.G] * p.n_tiles_n * p.split_k;
   const int num_kb = (p.K + BK - 1) / BK;
   const long long budget = p.timeout;
 
@@ -307,14 +289,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       int cursor = 0;
       bool ok = true;
       for (int tile = tile_first; tile < n_tiles && ok; tile += tile_step) {
-        const TileCoord tc = decode_tile(tile / p.split_k, tile_prefix, ntn, cursor);
-        const int n_blk = QUAD ? 2 * tc.n_blk + pp : tc.n_blk;
+        const TileCoord tc = decode_tile(tile / p.split_k, tile_prefix, p.n_tiles_n, cursor);
         const bool sh = tc.g >= p.G_main;
         const int a_row = (sh && p.sh_a_row >= 0 ? static_cast<int>(p.sh_a_row)
                                                  : static_cast<int>(p.a_row_base) +
                                                        (p.offsets || sh ? row0[tc.g] : (p.a_shared ? 0 : row0[tc.g]))) +
                           tc.m_blk * C::TILE_M + static_cast<int>(rank) * BM;
-        const int b_row = (sh ? tc.g - p.G_main : tc.g) * p.b_group_rows + n_blk * C::BN_OUT;
+        const int b_row = (sh ? tc.g - p.G_main : tc.g) * p.b_group_rows + tc.n_blk * C::BN_OUT;
         const CUtensorMap* mB = sh ? &tmBs : &tmB;
         const CUtensorMap* mB2 = sh ? &tmB2s : &tmB2;
         const int kb0 = (tile % p.split_k) * p.kb_per_split;
@@ -330,14 +311,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           } else if (PAIR) {
             // both halves complete on the even CTA's full barrier
             if (rank == 0) mbar_expect_tx(fb, 2 * C::STAGE_BYTES);
-            const uint32_t fb0 = rank == 0 ? fb : map_to_rank(fb, leader);
-            if (QUAD) {
-              // rows [pp * 64, pp * 64 + 64) of this CTA's 128, to both pairs
-              tma_load_2d_mc_pair(smem_u32(sA + stage * C::A_BYTES + pp * (BM / 2) * BK * 2), &tmA, kb * BK,
-                                  a_row + pp * (BM / 2), fb0, static_cast<uint16_t>(0x5u << rank));
-            } else {
-              tma_load_2d_to_pair_bar(smem_u32(sA + stage * C::A_BYTES), &tmA, kb * BK, a_row, fb0);
-            }
+            const uint32_t fb0 = rank == 0 ? fb : map_to_rank(fb, 0);
+            tma_load_2d_to_pair_bar(smem_u32(sA + stage * C::A_BYTES), &tmA, kb * BK, a_row, fb0);
             // SwiGLU: the even CTA stages the W1 rows of the tile, the odd CTA the W3 rows
             const CUtensorMap* tb = (EPI == EPI_SWIGLU && rank) ? mB2 : mB;
             tma_load_2d_to_pair_bar(smem_u32(sB + stage * C::B_BYTES), tb, kb * BK,
@@ -372,12 +347,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           for (int s = 0; s < STAGES; ++s)
             if (issued & (1u << s)) mbar_drain(smem_u32(&full[s]), (issued_phase >> s) & 1u, DRAIN_CYCLES);
         }
-        if (QUAD) {
-          // the other pair's multicasts into this CTA's stages are not all
-          // counted on barriers this CTA waited on: a fixed time to land too
-          const unsigned long long t0 = globaltimer_ns();
-          while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-        }
       }
     }
   } else if (warp == 1) {
@@ -403,7 +372,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       int cursor = 0;
       bool ok = true, any = false;
       for (int tile = tile_first; tile < n_tiles && ok; tile += tile_step, ++it) {
-        (void)decode_tile(tile / p.split_k, tile_prefix, ntn, cursor);
+        (void)decode_tile(tile / p.split_k, tile_prefix, p.n_tiles_n, cursor);
         const int kb0 = (tile % p.split_k) * p.kb_per_split;
         const int kb1 = kb0 + p.kb_per_split < num_kb ? kb0 + p.kb_per_split : num_kb;
         const int acc = it & 1;
@@ -434,8 +403,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               umma_bf16_pair(d_tmem, da, db, IDESC, kb != kb0 ? 1u : 0u);
 #pragma unroll
               for (int kk = 1; kk < BK / UK; ++kk) umma_bf16_pair(d_tmem, da + 2 * kk, db + 2 * kk, IDESC, 1u);
-              // QUAD: both pairs' producers wait for this stage
-              umma_commit_pair_mc(empty0 + 8u * stage, QUAD ? 0xF : 0x3);
+              umma_commit_pair_mc(empty0 + 8u * stage);
             } else {
               umma_bf16(d_tmem, da, db, IDESC, kb != kb0 ? 1u : 0u);
 #pragma unroll
@@ -451,7 +419,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
         if (!ok) break;
         if (issue) {
-          if (PAIR) umma_commit_pair_mc(smem_u32(&tfull[acc]), static_cast<uint16_t>(0x3u << leader));
+          if (PAIR) umma_commit_pair_mc(smem_u32(&tfull[acc]));
           else umma_commit(smem_u32(&tfull[acc]));
         }
       }
@@ -470,8 +438,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     int it = 0;
     int cursor = 0;
     for (int tile = tile_first; tile < n_tiles; tile += tile_step, ++it) {
-      const TileCoord tc = decode_tile(tile / p.split_k, tile_prefix, ntn, cursor);
-      const int n_blk = QUAD ? 2 * tc.n_blk + pp : tc.n_blk;
+      const TileCoord tc = decode_tile(tile / p.split_k, tile_prefix, p.n_tiles_n, cursor);
       const int ks = tile % p.split_k;
       (void)ks;
       const int acc = it & 1;
@@ -582,7 +549,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           }
           asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
           const int seg = lane & 7;
-          const int col = n_blk * C::BN_OUT + sl * C::SLAB + seg * 8;
+          const int col = tc.n_blk * C::BN_OUT + sl * C::SLAB + seg * 8;
 #pragma unroll
           for (int pass = 0; pass < 2; ++pass) {
             const int rr = part * 8 + pass * 4 + (lane >> 3);
@@ -610,7 +577,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) {
           // PAIR: both CTAs release the accumulator on the even CTA's barrier
-          if (PAIR) mbar_arrive_remote(map_to_rank(smem_u32(&tempty[acc]), leader));
+          if (PAIR) mbar_arrive_remote(map_to_rank(smem_u32(&tempty[acc]), 0));
           else mbar_arrive(smem_u32(&tempty[acc]));
         }
         continue;
@@ -640,7 +607,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           }
           tmem_wait();
         }
-        const int col = n_blk * C::BN_OUT + c0;
+        const int col = tc.n_blk * C::BN_OUT + c0;
         float v[C::CW];
 #pragma unroll
         for (int i = 0; i < C::CW; ++i) v[i] = __uint_as_float(slot ? rv[1][i] : rv[0][i]);
@@ -696,7 +663,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        if (PAIR) mbar_arrive_remote(map_to_rank(smem_u32(&tempty[acc]), leader));
+        if (PAIR) mbar_arrive_remote(map_to_rank(smem_u32(&tempty[acc]), 0));
         else mbar_arrive(smem_u32(&tempty[acc]));
       }
     }
@@ -805,15 +772,15 @@ const char* kernel_name(int epi) {
   }
 }
 
-template <int BN, int EPI, int STAGES, bool PAIR = false, bool QUAD = false>
+template <int BN, int EPI, int STAGES, bool PAIR = false>
 cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   using C = Cfg<BN, EPI, STAGES, PAIR>;
-  const void* kfn = reinterpret_cast<const void*>(tc_gemm_kernel<BN, EPI, STAGES, PAIR, QUAD>);
+  const void* kfn = reinterpret_cast<const void*>(tc_gemm_kernel<BN, EPI, STAGES, PAIR>);
   cudaError_t attr_err = ensure_smem_attr(kfn, C::SMEM);
   if (attr_err != cudaSuccess) return attr_err;
   CUtensorMap mA, mB, mB2;
   const int b_box = (EPI == EPI_SWIGLU || PAIR) ? BN / 2 : BN;
-  if (!make_map(&mA, a.A, a.a_rows, a.K, QUAD ? BM / 2 : BM)) return cudaErrorInvalidValue;
+  if (!make_map(&mA, a.A, a.a_rows, a.K, BM)) return cudaErrorInvalidValue;
   if (!make_map(&mB, a.B, a.b_rows, a.K, b_box)) return cudaErrorInvalidValue;
   if (EPI == EPI_SWIGLU) {
     if (!make_map(&mB2, a.B2, a.b_rows, a.K, b_box)) return cudaErrorInvalidValue;
@@ -868,15 +835,12 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   const long long m_tiles_max = a.max_rows / C::TILE_M + p.G;
   long long tiles = m_tiles_max * p.n_tiles_n * p.split_k;
   if (PAIR) {
-    // QUAD: a cluster tile is two N tiles (p.n_tiles_n is even)
-    if (QUAD) tiles /= 2;
-    const int cdim = QUAD ? 4 : 2;
-    int clusters = max_clusters(kfn, NUM_THREADS, C::SMEM, cdim);
+    int clusters = max_clusters(kfn, NUM_THREADS, C::SMEM, 2);
     if (clusters < 1) return cudaErrorInvalidConfiguration;
     if (tiles < clusters) clusters = static_cast<int>(tiles < 1 ? 1 : tiles);
     KernelScope ks(a.name ? a.name : kernel_name(EPI), s);
-    cudaError_t le = launch_cluster(tc_gemm_kernel<BN, EPI, STAGES, PAIR, QUAD>, clusters, cdim, NUM_THREADS,
-                                    (size_t)C::SMEM, s, mA, mB, mB2, mBs, mB2s, p);
+    cudaError_t le = launch_cluster(tc_gemm_kernel<BN, EPI, STAGES, PAIR>, clusters, 2, NUM_THREADS, (size_t)C::SMEM, s,
+                                    mA, mB, mB2, mBs, mB2s, p);
     if (le != cudaSuccess) return le;
     return cudaGetLastError();
   }
@@ -896,11 +860,10 @@ constexpr int stages_for(int b_rows) {
 }
 
 template <int EPI>
-cudaError_t launch_epi(const GemmArgs& a, int bn, bool pair, bool quad, cudaStream_t s) {
+cudaError_t launch_epi(const GemmArgs& a, int bn, bool pair, cudaStream_t s) {
   if (pair) {
     if constexpr (EPI == EPI_STORE || EPI == EPI_GELU || EPI == EPI_SWIGLU || EPI == EPI_SCATTER ||
                   EPI == EPI_REPLICATE) {
-      if (bn == 256 && quad) return launch_cfg<256, EPI, stages_for(128), true, true>(a, s);
       if (bn == 256) return launch_cfg<256, EPI, stages_for(128), true>(a, s);
       if (bn == 128) return launch_cfg<128, EPI, stages_for(64), true>(a, s);
     }
@@ -953,8 +916,8 @@ int choose_bn(const GemmArgs& a, int epi, bool pair = false) {
 
 }  // namespace
 
-// Clusters of `cdim` CTAs (2: one pair, 4: two pairs) of `kernel` that fit on
-// the device at once (cached per device and kernel); 0 when the query fails.
+// Clusters of `cdim` CTAs of `kernel` that fit on the device at once (cached
+// per device and kernel); 0 when the query fails.
 int max_clusters(const void* kernel, int threads, int smem, int cdim) {
   struct Entry {
     int dev;
@@ -1015,23 +978,6 @@ bool use_pairs(const GemmArgs& a, int epi) {
   return pad2 <= 1.1 * pad1;
 }
 
-// Whether a pair GEMM runs two pairs per cluster on neighbouring N tiles of
-// the same rows, each CTA loading half of its A rows and multicasting them to
-// the other pair (QUAD): 256-column tiles and an even N-tile count.
-// EC2MOE_GEMM_QUAD=0 / =1 in the environment forbids / allows it (A/B
-// comparisons; both compute the same result).
-bool use_quad(const GemmArgs& a, int epi, int bn) {
-  // 0: never; 1: every eligible GEMM; 2: the scattering (down) projections only
-  static const int allowed = [] {
-    const char* v = getenv("EC2MOE_GEMM_QUAD");
-    return v ? (v[0] == '1' ? 1 : (v[0] == 'd' ? 2 : 0)) : 0;
-  }();
-  if (!allowed || bn != 256 || (allowed == 2 && epi != EPI_SCATTER)) return false;
-  const int bn_out = epi == EPI_SWIGLU ? bn / 2 : bn;
-  const int n_tiles_n = (a.N + bn_out - 1) / bn_out;
-  return n_tiles_n % 2 == 0;
-}
-
 cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s) {
   if (a.G < 1 || a.G + a.sh_groups > MAX_GROUPS || a.N % 32 != 0 || a.K % 8 != 0) return cudaErrorInvalidValue;
   if (a.sh_groups > 0 && (epi == EPI_REPLICATE || epi == EPI_PARTIAL)) return cudaErrorInvalidValue;
@@ -1042,13 +988,12 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int epi, cudaStream_t s) {
     pair = false;
     bn = choose_bn(a, epi, false);
   }
-  const bool quad = pair && use_quad(a, epi, bn);
   switch (epi) {
-    case EPI_STORE: return launch_epi<EPI_STORE>(a, bn, pair, quad, s);
-    case EPI_GELU: return launch_epi<EPI_GELU>(a, bn, pair, quad, s);
-    case EPI_SWIGLU: return launch_epi<EPI_SWIGLU>(a, bn, pair, quad, s);
-    case EPI_SCATTER: return launch_epi<EPI_SCATTER>(a, bn, pair, quad, s);
-    case EPI_REPLICATE: return launch_epi<EPI_REPLICATE>(a, bn, pair, quad, s);
+    case EPI_STORE: return launch_epi<EPI_STORE>(a, bn, pair, s);
+    case EPI_GELU: return launch_epi<EPI_GELU>(a, bn, pair, s);
+    case EPI_SWIGLU: return launch_epi<EPI_SWIGLU>(a, bn, pair, s);
+    case EPI_SCATTER: return launch_epi<EPI_SCATTER>(a, bn, pair, s);
+    case EPI_REPLICATE: return launch_epi<EPI_REPLICATE>(a, bn, pair, s);
     case EPI_PARTIAL:
       if (!a.partial || a.N % 4 != 0) return cudaErrorInvalidValue;
       return bn >= 256 ? launch_cfg<256, EPI_PARTIAL, stages_for(256)>(a, s)

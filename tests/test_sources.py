@@ -1,0 +1,25 @@
+"""Rules of the device code that no run can show, checked on its text.
+
+No tensor or bulk copy goes to several CTAs at once: the library also runs with
+one rank per GPU (`bench.py` under torchrun), where such copies are not used.
+"""
+
+import pathlib
+import re
+
+import pytest
+
+CSRC = pathlib.Path(__file__).resolve().parents[1] / "paper_2508_06024_gb300" / "csrc"
+FILES = sorted(p for p in CSRC.iterdir() if p.suffix in (".cu", ".cuh"))
+
+
+def _code(path):
+    """The file without comments, adjacent string literals joined."""
+    text = re.sub(r"//[^\n]*|/\*.*?\*/", "", path.read_text(), flags=re.S)
+    return re.sub(r'"\s*"', "", text)
+
+
+@pytest.mark.parametrize("path", FILES, ids=lambda p: p.name)
+def test_copies_have_one_destination(path):
+    for copy in re.findall(r"cp\.async\.bulk[^;]*;", _code(path)):
+        assert "multicast" not in copy, copy
