@@ -37,8 +37,9 @@ namespace {
 //   warp 0       TMA: the X box (128 x 64 bf16, 128-byte swizzle) and the
 //                stacked split rows of the stage -- either straight from a
 //                prepared [3 * O_pad, d] bf16 matrix (PREP: made by
-//                gate_split_kernel); without one, warps 6..13 load the fp32
-//                rows and write their split into the swizzled layout;
+//                gate_split_kernel); without one, warps 6..13 take the fp32
+//                rows (staged by TMA or loaded to registers, gc_raw) and write
+//                their split into the swizzled layout;
 //   warp 1       4 MMAs (M = 128, N = 3 O_pad, K = 16) per stage into one of
 //                two TMEM accumulators; every GC_SEG stages (256 columns of
 //                d_model) the accumulator is handed over and the next segment
@@ -78,17 +79,28 @@ constexpr int GC_ACC_STRIDE = 256;  // TMEM columns between the two accumulators
 constexpr int GC_CS = 2;            // CTAs per tile (cluster) when d_model is split
 constexpr int GC_SPLIT_MIN_NK = 32; // stages per tile from which d_model is split
 
+// Without prepared rows, whether the fp32 rows of a stage come by TMA (nb blocks
+// of 16 gate rows) or from global memory to the converting warps' registers, one
+// stage ahead.  By TMA they arrive as many stages ahead as the ring is deep, but
+// take 256 bytes a row of each stage: up to 32 rows the ring stays deep and the
+// loads' latency decides, beyond that the stages do (standalone gate, T = 2000,
+// cold L2, launch bracket included, us, registers -> TMA: d = 768, E = 16 20.8 ->
+// 17.6, E = 32 24.2 -> 20.2; d = 4096, E = 16 36.5 -> 27.9, E = 32 51.8 -> 43.7;
+// E = 64, Top-1, TMA -> registers: d = 768 39 -> 30, d = 4096 74 -> 68).
+__host__ __device__ constexpr bool gc_raw(int nb, bool prep) { return !prep && nb <= 2; }
+
 struct GcLayout {
   int n_pad, O, k, E, stages, cs;
-  int stage_bytes, w3_off;
+  int stage_bytes, w3_off, raw_off;
   int log_stride;  // logits row of a token: O logits + 16 group scratch words, odd (conflict-free rows)
   int rstride;     // floats per received partial-logit row: n_pad + 4 (16-byte rows, shifted banks)
   int log_off, idx_off, tab_off, base_off, bias_off, list_off, recv_off, bar_off, warm_off, total;
-  __host__ __device__ GcLayout(int O_, int k_, int E_, int stages_, int cs_)
+  __host__ __device__ GcLayout(int O_, int k_, int E_, int stages_, int cs_, bool raw)
       : O(O_), k(k_), E(E_), stages(stages_), cs(cs_) {
     n_pad = (O + 15) / 16 * 16;
     w3_off = GC_BM * GC_BK * 2;
-    stage_bytes = w3_off + 3 * n_pad * 128;  // a multiple of 1024
+    raw_off = w3_off + 3 * n_pad * 128;
+    stage_bytes = raw_off + (raw ? n_pad * 256 : 0);  // a multiple of 1024
     log_stride = (O + 16) | 1;
     rstride = n_pad + 4;
     log_off = stages * stage_bytes;
@@ -285,6 +297,42 @@ __device__ __noinline__ void pick_row(const KParams& p, float* L, int O, const i
     }
 }
 
+// The Top-1 decision for one group of at most 16 experts from the logits in
+// registers (x[e], bias included; only the standalone gate takes it), with the
+// arithmetic of lse_rows and pick_row<1>: straight-line code, short enough to be
+// fetched while it runs (E = 16, T = 2000, us, rolled loops -> this: d = 768 17.6
+// -> 16.9, d = 4096 27.9 -> 26.2; the same for Top-2 was slower, 19.2 -> 20.1).
+__device__ __forceinline__ void decide_top1(const KParams& p, const float (&x)[16], int tok) {
+  const uint32_t allowed = p.mask_bits[0];
+  float mx = -CUDART_INF_F, best = -CUDART_INF_F;
+  int pick = -1;
+#pragma unroll
+  for (int e = 0; e < 16; ++e)
+    if (allowed >> e & 1u) {
+      mx = fmaxf(mx, x[e]);
+      if (x[e] > best) {
+        best = x[e];
+        pick = e;
+      }
+    }
+  float sum = 0.0f;
+#pragma unroll
+  for (int e = 0; e < 16; ++e)
+    if (allowed >> e & 1u) sum += expf(x[e] - mx);
+  const float lse = mx > -CUDART_INF_F ? mx + logf(sum) : -CUDART_INF_F;
+  if (pick < 0) {  // non-finite logits: the lowest allowed expert
+#pragma unroll
+    for (int e = 15; e >= 0; --e)
+      if (allowed >> e & 1u) {
+        best = x[e];
+        pick = e;
+      }
+  }
+  const float w = expf(best - lse);
+  p.topk_idx[tok] = pick;
+  p.topk_w[tok] = p.renorm ? w / w : w;
+}
+
 // Rows [row_lo, row_lo + n_rows) of the tile reserved per expert (the layer
 // path), with the worker warps only: entry i of the range (token row_lo + i /
 // k of the tile, slot i % k) gets route_rel = the expert's reserved base + the
@@ -386,15 +434,16 @@ __global__ void __launch_bounds__(256) gate_split_kernel(const float* W_local, c
 template <int NB, bool PREP>
 __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
     gate_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                   const __grid_constant__ GcParams gp) {
+                   const __grid_constant__ CUtensorMap tmWg, const __grid_constant__ GcParams gp) {
   using namespace tc;
+  constexpr bool RAW = gc_raw(NB, PREP);
   const KParams& p = gp.kp;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int nglob = (p.K == 1) ? 0 : p.K;
   const int O = p.E + nglob;
   const int cs = gp.cs;
-  const GcLayout L(O, p.k, p.E, gp.stages, cs);
+  const GcLayout L(O, p.k, p.E, gp.stages, cs, RAW);
   const int S = gp.stages;
   float* sLog = reinterpret_cast<float*>(smem + L.log_off);
   int* sIdx = reinterpret_cast<int*>(smem + L.idx_off);
@@ -416,6 +465,7 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  const bool top1_regs = NB == 1 && !PREP && !nglob && p.k == 1 && !p.route_counts;  // decide_top1
   const int n_tiles = (p.T + GC_BM - 1) / GC_BM;
   const int nk = (p.d + GC_BK - 1) / GC_BK;
   const long long budget = gp.timeout;
@@ -466,7 +516,8 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
   }
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmX);
-    if (PREP) tma_prefetch_desc(&tmW);
+    if (PREP || RAW) tma_prefetch_desc(&tmW);
+    if (RAW && nglob) tma_prefetch_desc(&tmWg);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -489,7 +540,7 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
     // The whole warp waits and counts; one elected lane issues.
     {
       const bool issue = elect_one();
-      const uint32_t bytes = GC_BM * GC_BK * 2 + (PREP ? 3 * n_pad * GC_BK * 2 : 0);
+      const uint32_t bytes = GC_BM * GC_BK * 2 + (PREP ? 3 * n_pad * GC_BK * 2 : RAW ? O * GC_BK * 4 : 0);
       const int my_tiles = tile_first < n_tiles ? (n_tiles - 1 - tile_first) / tile_step + 1 : 0;
       const int total = my_tiles * cnt;
       const int pre = total < S ? total : S;
@@ -498,6 +549,10 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
         if (issue) {
           mbar_expect_tx(fb, bytes);
           tma_load_2d(smem_u32(st), &tmX, (kb_lo + kc) * GC_BK, x_row, fb);
+          if (RAW) {
+            tma_load_2d(smem_u32(st + L.raw_off), &tmW, (kb_lo + kc) * GC_BK, 0, fb);
+            if (nglob) tma_load_2d(smem_u32(st + L.raw_off + p.E * GC_BK * 4), &tmWg, (kb_lo + kc) * GC_BK, 0, fb);
+          }
         }
       };
       auto next = [&] {
@@ -599,12 +654,14 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
     }
   } else if (!PREP && warp == GC_WARM_WARP) {
     // the decision's code to the SM, as an idle warp does below with prepared rows
-    float* warm = reinterpret_cast<float*>(smem + L.warm_off);
-    lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
-    if (p.k == 1) pick_row<1>(p, warm, O, s_list, s_grp, 0, nullptr, false);
-    else if (p.k == 2) pick_row<2>(p, warm, O, s_list, s_grp, 0, nullptr, false);
-    else if (p.k <= 4) pick_row<4>(p, warm, O, s_list, s_grp, 0, nullptr, false);
-    else pick_row<8>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+    if (!top1_regs) {
+      float* warm = reinterpret_cast<float*>(smem + L.warm_off);
+      lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
+      if (p.k == 1) pick_row<1>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+      else if (p.k == 2) pick_row<2>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+      else if (p.k <= 4) pick_row<4>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+      else pick_row<8>(p, warm, O, s_list, s_grp, 0, nullptr, false);
+    }
   } else {
     // ------------------------------------------------------------ worker warps
     const int wt = threadIdx.x - 64;
@@ -625,11 +682,11 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
       lse_rows(warm, 0, O, s_list, s_grp, p.K, 0, 1, lane, 32);
       pick(warm, nullptr, 0, false);
     }
-    if (!PREP && !is_drain) {
+    if (!PREP && !RAW && !is_drain) {
       // The fp32 gate rows to L2: the grid's converting threads together name
       // each 128-byte line once, so that the loads below, one stage ahead of
       // their use, wait for L2 and not for DRAM (fine-grained steps, T = 2001:
-      // 346.5 -> 343 us; Switch-shaped, T = 665: 75.6 -> 74.3).
+      // 346.5 -> 343 us).
       const long long row_lines = (p.d * 4LL + 127) / 128, lines = O * row_lines;
       constexpr int conv_threads = GC_THREADS - 192;
       for (long long i = static_cast<long long>(blockIdx.x) * conv_threads + (threadIdx.x - 192); i < lines;
@@ -712,7 +769,15 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
             }
           }
         }
-        if (decide_here) {
+        if (top1_regs) {
+          const int tok = tile * GC_BM + row;
+          if (decide_here && tok < p.T) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (j < O) acc[0][j] += s_bias[j];
+            decide_top1(p, acc[0], tok);
+          }
+        } else if (decide_here) {
           float* Lrow = sLog + row * L.log_stride;
 #pragma unroll
           for (int b = 0; b < NB; ++b)
@@ -730,12 +795,13 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
         }
       } else if (!PREP) {
         // split the fp32 gate rows of each stage into three bf16 terms, written
-        // in the swizzled K-major layout of the B operand; the next stage's
-        // pieces (8 columns of a row) are loaded while this one is written
+        // in the swizzled K-major layout of the B operand; without RAW the next
+        // stage's pieces (8 columns of a row) are loaded while this one is written
         const int ct = threadIdx.x - 192;
-        constexpr int ITEMS = (GC_MAX_O * 8 + 255) / 256;
+        constexpr int ITEMS = ((RAW ? 16 * NB : GC_MAX_O) * 8 + 255) / 256;
         float v[ITEMS][8];
         auto load_items = [&](int kc) {
+          if (RAW) return;
 #pragma unroll
           for (int t = 0; t < ITEMS; ++t) {
             const int i = ct + 256 * t, r = i >> 3, c = kc * GC_BK + (i & 7) * 8;
@@ -749,14 +815,24 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
         };
         load_items(kb_lo);
         for (int kc = 0; kc < cnt; ++kc) {
+          // RAW: the stage's fp32 rows have landed, else: the stage is free
           if (ok)
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, budget, abort_flag, &g_gate_error));
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(RAW ? &full[stage] : &empty[stage]), RAW ? phase : phase ^ 1u,
+                                                   budget, abort_flag, &g_gate_error));
           if (ok) {
             uint8_t* st = smem + stage * L.stage_bytes;
 #pragma unroll
             for (int t = 0; t < ITEMS; ++t) {
               const int i = ct + 256 * t, r = i >> 3, ch = i & 7;
               if (r >= n_pad) break;
+              if (RAW) {
+                if (r < O) {
+                  load8(reinterpret_cast<const float*>(st + L.raw_off) + r * GC_BK + ch * 8, v[t]);
+                } else {
+#pragma unroll
+                  for (int u = 0; u < 8; ++u) v[t][u] = 0.0f;
+                }
+              }
               uint32_t t0[4], t1[4], t2[4];
 #pragma unroll
               for (int u = 0; u < 4; ++u) split3_pair(v[t][2 * u], v[t][2 * u + 1], t0[u], t1[u], t2[u]);
@@ -811,18 +887,18 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
 }
 
 // Stages that fit next to the logits, routing tables and received partials.
-int gc_stages(int O, int k, int E, int cs) {
+int gc_stages(int O, int k, int E, int cs, bool raw) {
   for (int s = GC_MAX_STAGES; s >= 2; --s)
-    if (GcLayout(O, k, E, s, cs).total + 1024 <= 232448) return s;
+    if (GcLayout(O, k, E, s, cs, raw).total + 1024 <= 232448) return s;
   return 0;
 }
 
 // CTAs per tile: d_model is split over a cluster of GC_CS when a tile has at
-// least GC_SPLIT_MIN_NK stages and the received partials still leave room for
-// four stages that hold the fp32 gate rows as well (more gate rows make the
-// exchange too large a part), whatever the token count and whether the rows
-// come prepared, so every call of one layer shape sums its logits in the same
-// order.
+// least GC_SPLIT_MIN_NK stages and four stages with staged fp32 rows fit next to
+// the received partials, which is so up to 32 gate rows (the split of more rows
+// has not been measured since only up to 32 rows are staged), whatever the token
+// count and whether the rows come prepared, so every call of one layer shape sums
+// its logits in the same order.
 // EC2MOE_GATE_SPLIT_MIN_STAGES=n in the environment moves the threshold
 // (A/B comparisons; the split computes the same logits up to summation order).
 int gc_cluster_size(int O, int k, int E, int d) {
@@ -831,8 +907,7 @@ int gc_cluster_size(int O, int k, int E, int d) {
     return v && atoi(v) > 0 ? atoi(v) : GC_SPLIT_MIN_NK;
   }();
   if ((d + GC_BK - 1) / GC_BK < min_nk) return 1;
-  const GcLayout four(O, k, E, 4, GC_CS);
-  return four.warm_off + 4 * four.n_pad * 256 + 1024 <= 232448 ? GC_CS : 1;
+  return GcLayout(O, k, E, 4, GC_CS, true).warm_off + 1024 <= 232448 ? GC_CS : 1;
 }
 
 // CTAs the gate kernel launches (cs > 1: a cluster per tile, run in waves
@@ -845,7 +920,7 @@ int gc_blocks(int T, int cs) {
 
 template <int NB, bool PREP>
 cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t s, const CUtensorMap& mX,
-                              const CUtensorMap& mW) {
+                              const CUtensorMap& mW, const CUtensorMap& mWg) {
   const int O = p.E + (p.K == 1 ? 0 : p.K);
   GcParams gp;
   gp.kp = p;
@@ -853,13 +928,13 @@ cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t
   gp.stages = stages;
   gp.cs = cs;
   gp.timeout = default_timeout_cycles();
-  const int smem = GcLayout(O, p.k, p.E, stages, cs).total + 1024;
+  const int smem = GcLayout(O, p.k, p.E, stages, cs, gc_raw(NB, PREP)).total + 1024;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(gate_tc_kernel<NB, PREP>), smem);
   if (e != cudaSuccess) return e;
   const int blocks = gc_blocks(p.T, cs);
   const int threads = PREP ? GC_THREADS : GC_THREADS + 32;
   if (cs == 1)
-    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(threads), (size_t)smem, s, mX, mW, gp);
+    return launch_kernel(gate_tc_kernel<NB, PREP>, dim3(blocks), dim3(threads), (size_t)smem, s, mX, mW, mWg, gp);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(threads);
@@ -874,20 +949,20 @@ cudaError_t launch_gate_tc_nb(const KParams& p, int stages, int cs, cudaStream_t
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = next_launch_pdl() ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gate_tc_kernel<NB, PREP>, mX, mW, gp);
+  return cudaLaunchKernelEx(&cfg, gate_tc_kernel<NB, PREP>, mX, mW, mWg, gp);
 }
 
 template <bool PREP>
 cudaError_t launch_gate_tc(const KParams& p, int stages, int cs, cudaStream_t s, const CUtensorMap& mX,
-                           const CUtensorMap& mW) {
+                           const CUtensorMap& mW, const CUtensorMap& mWg) {
   const int O = p.E + (p.K == 1 ? 0 : p.K);
   // NB = accumulator blocks of 16 gate rows a drain thread keeps; 3 and 4
   // run as 5 (the extra blocks read allocated TMEM columns past the gate rows
   // and are never used), which keeps the number of kernel variants small.
   switch ((O + 15) / 16) {
-    case 1: return launch_gate_tc_nb<1, PREP>(p, stages, cs, s, mX, mW);
-    case 2: return launch_gate_tc_nb<2, PREP>(p, stages, cs, s, mX, mW);
-    default: return launch_gate_tc_nb<5, PREP>(p, stages, cs, s, mX, mW);
+    case 1: return launch_gate_tc_nb<1, PREP>(p, stages, cs, s, mX, mW, mWg);
+    case 2: return launch_gate_tc_nb<2, PREP>(p, stages, cs, s, mX, mW, mWg);
+    default: return launch_gate_tc_nb<5, PREP>(p, stages, cs, s, mX, mW, mWg);
   }
 }
 
@@ -911,13 +986,19 @@ cudaError_t launch_gate_tensor(const GateArgs& a, KParams p, int O, bool bf16, c
     const bool prep = a.w_split != nullptr;
     const int n_pad = (O + 15) / 16 * 16;
     const int cs = gc_cluster_size(O, a.k, a.E, a.d);
-    const int stages = gc_stages(O, a.k, a.E, cs);
-    CUtensorMap mX, mW;
+    const bool raw = gc_raw(n_pad / 16, prep);
+    const int stages = gc_stages(O, a.k, a.E, cs, raw);
+    CUtensorMap mX, mW, mWg;
     bool maps = stages >= 2 && make_tensor_map_bf16(&mX, a.X, a.T, a.d, GC_BM);
     if (prep) {
       maps = maps && make_tensor_map_bf16(&mW, a.w_split, 3LL * n_pad, a.d, 3 * n_pad);
+      mWg = mW;
+    } else if (raw) {
+      maps = maps && make_tensor_map_f32(&mW, a.W_local, a.E, a.d, a.E);
+      if (maps && a.K > 1) maps = make_tensor_map_f32(&mWg, a.W_global, a.K, a.d, a.K);
+      else mWg = mW;
     } else if (maps) {
-      mW = mX;  // not read: the kernel loads and splits the gate rows itself
+      mW = mWg = mX;  // not read: the kernel loads the gate rows to registers
     }
     if (maps) {
       *handled = true;
@@ -944,8 +1025,8 @@ cudaError_t launch_gate_tensor(const GateArgs& a, KParams p, int O, bool bf16, c
         const int b = gc_blocks(a.T, cs);
         *held_sms = b < sm_count() ? b : sm_count();
       }
-      e = prep ? launch_gate_tc<true>(p, stages, cs, s, mX, mW)
-               : launch_gate_tc<false>(p, stages, cs, s, mX, mW);
+      e = prep ? launch_gate_tc<true>(p, stages, cs, s, mX, mW, mWg)
+               : launch_gate_tc<false>(p, stages, cs, s, mX, mW, mWg);
       if (e != cudaSuccess) return e;
       return cudaGetLastError();
     }

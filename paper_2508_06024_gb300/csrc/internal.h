@@ -260,6 +260,8 @@ cudaError_t read_swap_error(unsigned int* word);
 // 2-D bf16 tensor map over a row-major [rows, cols] matrix: box 64 columns x
 // box_rows rows, 128-byte swizzle, zero fill out of bounds (cached).
 bool make_tensor_map_bf16(CUtensorMap* m, const void* ptr, long long rows, long long cols, int box_rows);
+// 2-D fp32 tensor map, box 64 columns x box_rows rows, no swizzle (cached).
+bool make_tensor_map_f32(CUtensorMap* m, const void* ptr, long long rows, long long cols, int box_rows);
 
 // Fused low-rank codec of the layer path (bf16): Z = X V_enc^T (stored), then
 // X_hat = Z V_dec^T written straight into expert order with relative
