@@ -40,7 +40,9 @@
 //
 // A result that is not finite (an infinite or NaN operand, an operand that
 // rounds to infinity in bf16, an overflow) is computed again as the sequential
-// fp32 FMA sum: the split of an infinity has no exact terms.
+// fp32 FMA sum: the split of an infinity has no exact terms.  That is slow (the
+// layer above, 164 us eager: 202 with one infinite value in one row, 1015 with one
+// in every row; with one sum after the other 274 and 2119).
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -152,18 +154,44 @@ __device__ __forceinline__ void split3(const float4& v, uint2& t0, uint2& t1, ui
   split3(v.z, v.w, t0.y, t1.y, t2.y);
 }
 
-// One result as the sequential fp32 FMA sum (results that are not finite).
-// A sum that has become NaN stays NaN, so rows of NaNs end at once.
-__device__ __noinline__ float fma_dot(const float* a, const float* b, int K) {
-  float s = 0.0f;
-  for (int k = 0; k < K; k += 8) {  // K is a multiple of 8
-#pragma unroll
-    for (int u = 0; u < 8; ++u) s = fmaf(a[k + u], b[k + u], s);
-    if (s != s) break;
-  }
-  return s;
-}
 __device__ __forceinline__ bool finite(float v) { return fabsf(v) < __int_as_float(0x7f800000); }
+
+// Four neighbouring results (rows b, b + K, ... of the weights): those that are
+// not finite as sequential fp32 FMA sums, side by side, so that a row of
+// infinities waits for the loads of eight columns once and not once per result.
+// A sum that has become NaN stays NaN, so rows of NaNs end at once.
+__device__ __noinline__ float4 fma_redo(float4 v, const float* a, const float* b, int K) {
+  float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const bool redo[4] = {!finite(v.x), !finite(v.y), !finite(v.z), !finite(v.w)};
+#pragma unroll 2
+  for (int k = 0; k < K; k += 8) {  // K is a multiple of 8
+    float x[8], w[4][8];
+    load8(a + k, x);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) w[j][u] = 0.0f;
+      if (redo[j]) load8(b + (long long)j * K + k, w[j]);
+    }
+    bool open = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s[j] = fmaf(x[u], w[j][u], s[j]);
+      open |= redo[j] && s[j] == s[j];
+    }
+    if (!open) break;
+  }
+  return make_float4(redo[0] ? s[0] : v.x, redo[1] ? s[1] : v.y, redo[2] ? s[2] : v.z, redo[3] ? s[3] : v.w);
+}
+__device__ __forceinline__ void make_finite(float (&v)[4], const float* a, const float* b, int K) {
+  if (finite(v[0]) && finite(v[1]) && finite(v[2]) && finite(v[3])) return;
+  const float4 r = fma_redo(make_float4(v[0], v[1], v[2], v[3]), a, b, K);
+  v[0] = r.x;
+  v[1] = r.y;
+  v[2] = r.z;
+  v[3] = r.w;
+}
 
 // A tile's place: group, valid rows and output columns, first rows of A and B.
 struct FTile {
@@ -355,14 +383,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
       const float* src_a =
           p.A + (tc.a_row + (arow_l < m_left && tc.a_row + arow_l < p.a_rows ? arow_l : 0)) * p.K + ac0;
       uint32_t live = 0;  // bit i: B piece i
-      const float* src_b[C::B_CHUNKS];
+      // rows 0 .. BN_OUT - 1 of the block from B, the rest (SwiGLU) from B2; 32-bit
+      // offsets, as registers are short
+      const float* src_b = p.B + tc.b_row * p.K + lc;
+      const float* src_b2 = GLU ? p.B2 + tc.b_row * p.K + lc : src_b;
+      int off_b[C::B_CHUNKS];
 #pragma unroll
       for (int i = 0; i < C::B_CHUNKS; ++i) {
-        // rows 0 .. BN_OUT - 1 of the block from B, the rest (SwiGLU) from B2
         const int r = (lr + 32 * i) % BN_OUT;
         const bool in = r < n_left;
         live |= in ? 1u << i : 0u;
-        src_b[i] = (GLU && 32 * i >= BN_OUT ? p.B2 : p.B) + (tc.b_row + (in ? r : 0)) * p.K + lc;
+        off_b[i] = (in ? r : 0) * p.K;
       }
       float ra[16];
       float4 rb[C::B_CHUNKS];
@@ -389,8 +420,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
       auto load_b = [&](int kb) {
         const bool in_k = kb * BK + lc < p.K;
 #pragma unroll
-        for (int i = 0; i < C::B_CHUNKS; ++i)
-          rb[i] = in_k ? __ldg(reinterpret_cast<const float4*>(src_b[i] + kb * BK)) : zero;
+        for (int i = 0; i < C::B_CHUNKS; ++i) {
+          const float* src = (GLU && 32 * i >= BN_OUT ? src_b2 : src_b) + off_b[i] + kb * BK;
+          rb[i] = in_k ? __ldg(reinterpret_cast<const float4*>(src)) : zero;
+        }
       };
       float acc[NC];
 #pragma unroll
@@ -522,16 +555,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
         float v[4], w[4];
         *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(tile_out + local * C::PITCH + c);
         if (GLU) *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(tile_out + local * C::PITCH + BN / 2 + c);
+        const float* arow = p.A + (tc.a_row + local) * p.K;
+        const long long brow = (tc.b_row + c) * p.K;
+        make_finite(v, arow, p.B + brow, p.K);
+        if (GLU) make_finite(w, arow, p.B2 + brow, p.K);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const float* arow = p.A + (tc.a_row + local) * p.K;
-          const long long brow = (tc.b_row + c + u) * p.K;
-          if (!finite(v[u])) v[u] = fma_dot(arow, p.B + brow, p.K);
           if (EPI == EPI_GELU) v[u] = gelu_erf(v[u]);
-          if (GLU) {
-            if (!finite(w[u])) w[u] = fma_dot(arow, p.B2 + brow, p.K);
-            v[u] = silu(v[u]) * w[u];
-          }
+          if (GLU) v[u] = silu(v[u]) * w[u];
           if (EPI == EPI_SCATTER) v[u] *= sc;
         }
         const float4 o = make_float4(v[0], v[1], v[2], v[3]);

@@ -103,3 +103,19 @@ def test_f32_nonfinite_results_follow_the_fma_sum():
     assert bool(Z[4].isnan().all())
     keep = [i for i in range(130) if i not in (3, 4)]
     _check(Z[keep], X[keep], V)
+
+
+def test_f32_recomputes_single_results():
+    """One infinite weight in some of four neighbouring columns, which are
+    computed again together: the finite ones keep their bits."""
+    X, V = _randn(1, 130, 136), _randn(2, 72, 136)
+    desc = C.make_desc(T=130, d=136, E=8, d_ff=8, k=1, dtype=C.F32, r=72)
+    Z, ref = torch.empty(130, 72, device="cuda"), torch.empty(130, 72, device="cuda")
+    C.ec2moe_lr_encode(desc, X, V, ref)
+    bad = [1, 3, 40, 68, 69, 70, 71]
+    V[bad, 135] = float("inf")
+    C.ec2moe_lr_encode(desc, X, V, Z)
+    assert C.ec2moe_last_device_error() == C.OK
+    good = [i for i in range(72) if i not in bad]
+    assert torch.equal(Z[:, good], ref[:, good])
+    assert torch.equal(Z[:, bad], (torch.sign(X[:, 135:]) * float("inf")).expand(130, len(bad)))
