@@ -9,7 +9,12 @@
 // below 2^-26 |x|).  A product of two bf16 terms is exact in fp32, and
 //   x w = x0 w0 + (x0 w1 + x1 w0) + (x0 w2 + x1 w1 + x2 w0) + rest,
 // with a rest of at most about 2^-25 |x w|, under one fp32 rounding of the
-// product.  The tensor core adds into its fp32 accumulator without rounding to
+// product.  bf16 ends 16 binary places before fp32, and the tensor core reads
+// subnormal operands as 0, so operands are scaled by 2^24 first (exact), which
+// keeps that true down to fp32's smallest numbers.  What the scaling makes
+// overflow (operands above 2^104, sums above 2^80) is computed again, see below.
+//
+// The tensor core adds into its fp32 accumulator without rounding to
 // nearest, so sums are kept short: x0 w0 accumulates in one TMEM accumulator
 // and the five smaller products in another, both only over a segment of 128
 // columns of K; the warps then add the two and the segment's sum to fp32
@@ -38,9 +43,9 @@
 // stages take the other pair's columns).  Every wait is bounded; a timeout sets
 // the error word and the CTA ends after its MMAs in flight.
 //
-// A result that is not finite (an infinite or NaN operand, an operand that
-// rounds to infinity in bf16, an overflow) is computed again as the sequential
-// fp32 FMA sum: the split of an infinity has no exact terms.  That is slow (the
+// A result that is not finite (an infinite or NaN operand, an overflow of a
+// scaled operand or sum) is computed again as the sequential fp32 FMA sum: the
+// split of an infinity has no exact terms.  That is slow (the
 // layer above, 164 us eager: 202 with one infinite value in one row, 1015 with one
 // in every row; with one sum after the other 274 and 2119).
 #include <cuda_runtime.h>
@@ -138,8 +143,21 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   return r;
 }
 
-// The three bf16 terms of two fp32 values.
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// Every operand is multiplied by SCALE before it is split, every sum by UNSCALE
+// after: with the last bit of an fp32 number at 2^-149 or above, all its terms
+// are then normal bf16 numbers.
+constexpr float SCALE = 0x1p24f;
+constexpr float UNSCALE = 0x1p-48f;
+
+// The three bf16 terms of two fp32 values, scaled.
 __device__ __forceinline__ void split3(float x, float y, uint32_t& t0, uint32_t& t1, uint32_t& t2) {
+  unpack2(mul2(pack2(x, y), pack2(SCALE, SCALE)), x, y);
   t0 = pack_bf16x2(x, y);
   const uint64_t r1 = sub2(pack2(x, y), pack2(bf16_lo(t0), bf16_hi(t0)));
   float a, b;
@@ -156,8 +174,8 @@ __device__ __forceinline__ void split3(const float4& v, uint2& t0, uint2& t1, ui
 
 __device__ __forceinline__ bool finite(float v) { return fabsf(v) < __int_as_float(0x7f800000); }
 
-// Four neighbouring results (rows b, b + K, ... of the weights): those that are
-// not finite as sequential fp32 FMA sums, side by side, so that a row of
+// Four neighbouring results (rows b, b + K, ... of the weights) from their scaled
+// sums: those that are not finite as sequential fp32 FMA sums, side by side, so that a row of
 // infinities waits for the loads of eight columns once and not once per result.
 // A sum that has become NaN stays NaN, so rows of NaNs end at once.
 __device__ __noinline__ float4 fma_redo(float4 v, const float* a, const float* b, int K) {
@@ -182,10 +200,15 @@ __device__ __noinline__ float4 fma_redo(float4 v, const float* a, const float* b
     }
     if (!open) break;
   }
-  return make_float4(redo[0] ? s[0] : v.x, redo[1] ? s[1] : v.y, redo[2] ? s[2] : v.z, redo[3] ? s[3] : v.w);
+  return make_float4(redo[0] ? s[0] : v.x * UNSCALE, redo[1] ? s[1] : v.y * UNSCALE, redo[2] ? s[2] : v.z * UNSCALE,
+                     redo[3] ? s[3] : v.w * UNSCALE);
 }
-__device__ __forceinline__ void make_finite(float (&v)[4], const float* a, const float* b, int K) {
-  if (finite(v[0]) && finite(v[1]) && finite(v[2]) && finite(v[3])) return;
+__device__ __forceinline__ void finish(float (&v)[4], const float* a, const float* b, int K) {
+  if (finite(v[0]) && finite(v[1]) && finite(v[2]) && finite(v[3])) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] *= UNSCALE;
+    return;
+  }
   const float4 r = fma_redo(make_float4(v[0], v[1], v[2], v[3]), a, b, K);
   v[0] = r.x;
   v[1] = r.y;
@@ -557,8 +580,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
         if (GLU) *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(tile_out + local * C::PITCH + BN / 2 + c);
         const float* arow = p.A + (tc.a_row + local) * p.K;
         const long long brow = (tc.b_row + c) * p.K;
-        make_finite(v, arow, p.B + brow, p.K);
-        if (GLU) make_finite(w, arow, p.B2 + brow, p.K);
+        finish(v, arow, p.B + brow, p.K);
+        if (GLU) finish(w, arow, p.B2 + brow, p.K);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (EPI == EPI_GELU) v[u] = gelu_erf(v[u]);

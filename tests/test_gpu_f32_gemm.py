@@ -2,10 +2,10 @@
 of its tiles, against float64.
 
 Bound per element: every product is exact up to 2^-24 |a b| (the three-term
-split), a 64-column block adds 4 MMAs of 16 products into one accumulator and
-20 into the other without rounding to nearest (at most 2^-23 of the running
+split), a segment of 128 columns adds 8 MMAs of 16 products into one accumulator
+and 40 into the other without rounding to nearest (at most 2^-23 of the running
 magnitude per MMA; the second accumulator holds terms of 2^-8 |a b|), and the
-K / 64 blocks are added in fp32 (2^-24 each), so
+K / 128 segments are added in fp32 (2^-24 each), so
 |error| <= (8 + K / 64) 2^-23 sum_k |a_k b_k|.
 """
 
@@ -30,9 +30,9 @@ def _randn(seed, *shape):
     return torch.randn(*shape, generator=g, device="cuda")
 
 
-def _check(got, A, W):
+def _check(got, A, W, least=0.0):
     ref = A.double() @ W.double().T
-    bound = (8 + A.shape[1] / 64) * 2.0 ** -23 * (A.double().abs() @ W.double().abs().T)
+    bound = least + (8 + A.shape[1] / 64) * 2.0 ** -23 * (A.double().abs() @ W.double().abs().T)
     assert bool(((got.double() - ref).abs() <= bound).all())
 
 
@@ -119,3 +119,21 @@ def test_f32_recomputes_single_results():
     good = [i for i in range(72) if i not in bad]
     assert torch.equal(Z[:, good], ref[:, good])
     assert torch.equal(Z[:, bad], (torch.sign(X[:, 135:]) * float("inf")).expand(130, len(bad)))
+
+
+# Operands over the whole exponent range: near and below the smallest normal
+# number, products that small, and magnitudes whose scaled terms or sums
+# overflow and are computed again.  Products and sums are exact down to far
+# below fp32's smallest step, so the only absolute error is that of a result
+# stored as a subnormal number (half of 2^-149).
+@pytest.mark.parametrize("x2,w2", [(-120, 0), (0, -120), (-126, 10), (-140, 60), (-60, -60), (100, -100), (60, 30),
+                                   (110, -60), (-70, 110)])
+def test_f32_operand_range(x2, w2):
+    T, d, r = 130, 200, 72
+    X = (_randn(1, T, d).double() * 2.0 ** x2).float()
+    V = (_randn(2, r, d).double() * 2.0 ** w2).float()
+    desc = C.make_desc(T=T, d=d, E=8, d_ff=8, k=1, dtype=C.F32, r=r)
+    Z = torch.empty(T, r, device="cuda")
+    C.ec2moe_lr_encode(desc, X, V, Z)
+    assert C.ec2moe_last_device_error() == C.OK
+    _check(Z, X, V, 2.0 ** -149)
