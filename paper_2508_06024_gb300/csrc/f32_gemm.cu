@@ -41,7 +41,9 @@
 // Two stages, so a block is loaded and split while the previous one multiplies;
 // two pairs of accumulators for 64-wide tiles, one for 128-wide ones (the A
 // stages take the other pair's columns).  Every wait is bounded; a timeout sets
-// the error word and the CTA ends after its MMAs in flight.
+// the error word and the CTA ends after its MMAs in flight.  A comes by plain
+// loads: the kernel before may still write it when this one starts, which the
+// read-only path does not allow.
 //
 // A result that is not finite (an infinite or NaN operand, an overflow of a
 // scaled operand or sum) is computed again as the sequential fp32 FMA sum: the
@@ -430,12 +432,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
 #pragma unroll
             for (int u = 0; u < 8; ++u) r[u] = 0.0f;
           } else if (wide_a) {
-            asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                          : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
                          : "l"(src_a + kb * BK + h * 8));
           } else {
-            const float4 x = __ldg(reinterpret_cast<const float4*>(src_a + kb * BK + h * 8));
-            const float4 y = __ldg(reinterpret_cast<const float4*>(src_a + kb * BK + h * 8 + 4));
+            const float4 x = *reinterpret_cast<const float4*>(src_a + kb * BK + h * 8);
+            const float4 y = *reinterpret_cast<const float4*>(src_a + kb * BK + h * 8 + 4);
             r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w; r[4] = y.x; r[5] = y.y; r[6] = y.z; r[7] = y.w;
           }
         }

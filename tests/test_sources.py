@@ -2,6 +2,10 @@
 
 No tensor or bulk copy goes to several CTAs at once: the library also runs with
 one rank per GPU (`bench.py` under torchrun), where such copies are not used.
+
+The read-only load path is for weights alone: with programmatic dependent launch
+a kernel starts while the one before still writes its activations, and PTX allows
+read-only loads only of memory that nobody writes while the kernel runs.
 """
 
 import pathlib
@@ -23,3 +27,12 @@ def _code(path):
 def test_copies_have_one_destination(path):
     for copy in re.findall(r"cp\.async\.bulk[^;]*;", _code(path)):
         assert "multicast" not in copy, copy
+
+
+@pytest.mark.parametrize("path", FILES, ids=lambda p: p.name)
+def test_read_only_loads_are_of_weights(path):
+    code = _code(path)
+    assert not re.findall(r"\bld\.global[.\w]*\.nc\b", code)
+    lines = [line for line in code.splitlines() if "__ldg(" in line]
+    # the weight rows of the fp32 GEMM
+    assert all("rb[i]" in line for line in lines), lines
