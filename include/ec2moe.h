@@ -288,9 +288,11 @@ ec2moe_status ec2moe_last_device_error(ec2moe_stream_t stream);
  * wait that runs out makes its CTA stop, wait (with a fixed one-second
  * budget) for the copies and MMAs it started, free its tensor memory and
  * return; ec2moe_last_device_error then reports EC2MOE_ERR_TIMEOUT and the
- * context stays usable.  A budget of 0 makes every wait that is not already
- * satisfied give up at once, which is how failure handling is exercised
- * without a real fault.  Negative values return EC2MOE_ERR_INVALID_ARG. */
+ * context stays usable.  With a budget of 0 a wait gives up when the hardware's
+ * own try (which may suspend for a few microseconds) finds it unsatisfied, and
+ * the fp32 GEMM's waits for its accumulators at once; that is how failure
+ * handling is exercised without a real fault.  Negative values return
+ * EC2MOE_ERR_INVALID_ARG. */
 ec2moe_status ec2moe_set_wait_budget(int64_t cycles);
 int64_t ec2moe_get_wait_budget(void);
 

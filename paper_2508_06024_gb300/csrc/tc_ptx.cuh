@@ -56,6 +56,28 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
     }
   }
 }
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// The same, and with a budget of 0 it gives up on every barrier that is not
+// complete yet: a try may suspend the thread for microseconds, in which all the
+// waits of a kernel whose waits are short come to pass.
+__device__ __forceinline__ bool mbar_wait_strict(uint32_t bar, uint32_t parity, long long budget,
+                                                 volatile int* abort_flag, unsigned int* err_word) {
+  if (budget > 0) return mbar_wait(bar, parity, budget, abort_flag, err_word);
+  if (mbar_test_wait(bar, parity)) return true;
+  *abort_flag = 1;
+  atomicOr(err_word, 1u);
+  return false;
+}
 // Budget of the drain waits after an abort (about one second at the maximum
 // SM clock), independent of the caller-set wait budget: copies and MMAs a
 // CTA started must land before its shared memory and TMEM are released,

@@ -137,3 +137,31 @@ def test_f32_operand_range(x2, w2):
     C.ec2moe_lr_encode(desc, X, V, Z)
     assert C.ec2moe_last_device_error() == C.OK
     _check(Z, X, V, 2.0 ** -149)
+
+
+# Every kernel shape: 64- and 128-wide tiles, K split over a cluster and not,
+# one tile and several per CTA.  With a budget of 0 a wait that is not satisfied
+# at once gives up; the CTA still meets its cluster's barriers, ends its MMAs in
+# flight and returns, and the next call finds nothing left over.
+@pytest.mark.parametrize("T,d,r,decode", [(256, 512, 64, False), (4096, 768, 128, False), (300, 768, 128, True),
+                                          (4096, 768, 128, True)],
+                         ids=["64-wide-split", "128-wide-split", "64-wide", "128-wide"])
+def test_f32_zero_wait_budget_times_out_and_recovers(T, d, r, decode):
+    desc = C.make_desc(T=T, d=d, E=8, d_ff=8, k=1, dtype=C.F32, r=r)
+    A, W = _randn(1, T, r if decode else d), _randn(2, *((d, r) if decode else (r, d)))
+    call = C.ec2moe_lr_decode if decode else C.ec2moe_lr_encode
+    ref, out = torch.empty(T, W.shape[0], device="cuda"), torch.empty(T, W.shape[0], device="cuda")
+    call(desc, A, W, ref)
+    assert C.ec2moe_last_device_error() == C.OK
+    old = C.ec2moe_get_wait_budget()
+    try:
+        C.ec2moe_set_wait_budget(0)
+        call(desc, A, W, out)
+        status = C.ec2moe_last_device_error()
+    finally:
+        C.ec2moe_set_wait_budget(old)
+    assert status == C.ERR_TIMEOUT
+    assert C.ec2moe_last_device_error() == C.OK  # the error word was read and cleared
+    call(desc, A, W, out)
+    assert C.ec2moe_last_device_error() == C.OK
+    assert torch.equal(out, ref)
