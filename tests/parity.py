@@ -106,3 +106,16 @@ def output_check(y_gpu: np.ndarray, y_ref: np.ndarray, bf16: bool, pair: bool = 
     else:
         assert err <= 1e-4, f"relative Frobenius error {err:.3e} > 1e-4"
     return err, mx
+
+
+def gemm_launches(call, name):
+    """How many GEMM kernels called `name` the call launches; None where kernels
+    cannot be traced (a process's first trace may come back empty)."""
+    for _ in range(3):
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events() if "gemm_kernel" in e.name]
+        if names:
+            return sum(name in n for n in names)
+    return None

@@ -106,14 +106,14 @@ def test_route_out_of_range_ids_are_skipped_and_reported(T, k, E, noalloc):
 
 # Expert-order tables handed to ec2moe_experts that do not describe the call's
 # rows: every grouped GEMM (swapped-operand kernel for <= 16 rows, tensor-core
-# kernel, SIMT kernel for fp32) checks each group range against the rows and
+# kernel, fp32 kernel) checks each group range against the rows and
 # each scatter destination, skips what lies outside, and reports
 # EC2MOE_ERR_INVALID_ARG; nothing past the output buffer is written.
 EXPERT_SHAPES = [(8, 2, 4, 256, 256, C.BF16), (200, 2, 4, 256, 512, C.BF16), (96, 2, 4, 128, 256, C.F32)]
 CORRUPTIONS = ["offset-past-rows", "negative-offset", "decreasing-offsets", "perm-out-of-range"]
 
 
-@pytest.mark.parametrize("shape", EXPERT_SHAPES, ids=["swapped", "tensor-core", "simt-fp32"])
+@pytest.mark.parametrize("shape", EXPERT_SHAPES, ids=["swapped", "tensor-core", "fp32"])
 @pytest.mark.parametrize("bad", CORRUPTIONS)
 def test_experts_skip_tables_outside_the_rows(shape, bad):
     T, k, E, d, d_ff, dtype = shape

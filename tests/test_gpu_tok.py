@@ -14,7 +14,7 @@ import torch
 
 from paper_2508_06024_gb300 import build as B
 from paper_2508_06024_gb300 import ec2moe as C
-from tests.parity import rel_fro
+from tests.parity import gemm_launches, rel_fro
 
 pytestmark = pytest.mark.gpu
 
@@ -62,6 +62,7 @@ def _check_group(t, e, lo, hi, act, out):
 @pytest.mark.parametrize("rows", [[1, 257, 0, 800], [33, 256, 511, 288]], ids=["uneven", "edges"])
 def test_experts_tokens_on_n(rows, act, ff):
     t, off, desc, ws = _case(rows, 2592, ff, act, 7)
+    assert gemm_launches(lambda: _run(t, off, desc, ws), "tok_gemm_kernel") in (2, None)
     out = _run(t, off, desc, ws)
     assert C.ec2moe_last_device_error() == C.OK
     assert not bool(out.isnan().any())
