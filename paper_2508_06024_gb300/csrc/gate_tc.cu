@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
   }
   for (int o = threadIdx.x - 64; o >= 0 && o < O; o += PREP ? GC_THREADS - 64 : GC_THREADS - 32)
     s_bias[o] = o < p.E ? p.b_local[o] : p.b_global[o - p.E];
-  if (warp == 2) {
+  if (warp == 2 && !top1_regs) {
     // the allowed experts in ascending order, and where each group's begin
     const int gsize = p.E / p.K;
     int base = 0;
@@ -548,11 +548,11 @@ __global__ void __launch_bounds__(PREP ? GC_THREADS : GC_THREADS + 32, 1)
       auto load_x = [&](uint8_t* st, uint32_t fb) {
         if (issue) {
           mbar_expect_tx(fb, bytes);
-          tma_load_2d(smem_u32(st), &tmX, (kb_lo + kc) * GC_BK, x_row, fb);
-          if (RAW) {
+          if (RAW) {  // first: the rows are converted before X is multiplied
             tma_load_2d(smem_u32(st + L.raw_off), &tmW, (kb_lo + kc) * GC_BK, 0, fb);
             if (nglob) tma_load_2d(smem_u32(st + L.raw_off + p.E * GC_BK * 4), &tmWg, (kb_lo + kc) * GC_BK, 0, fb);
           }
+          tma_load_2d(smem_u32(st), &tmX, (kb_lo + kc) * GC_BK, x_row, fb);
         }
       };
       auto next = [&] {
