@@ -19,16 +19,16 @@
 // and the five smaller products in another, both only over a segment of 128
 // columns of K; the warps then add the two and the segment's sum to fp32
 // registers.  Against 64-bit results this is closer than the sequential fp32
-// FMA sums of a CUDA-core kernel: relative error of a layer's Y 5.1e-7
+// FMA sums of a CUDA-core kernel: relative error of a layer's Y 5.0e-7
 // against 1.3e-6 (d = 768, d_ff = 3072), 4.4e-7 against 8.7e-7 (512, 1024).
 //
 // What bounds it: a chain of nearly equal parts per 64-column block.  A pass of
 // a layer (12 experts, 1024 rows, 768 x 3072; the two expert GEMMs are 4/5 of
-// it) takes 155 us, copies of the kernel without the MMAs 128, with half of
-// them 133, without B's split and stores 142, without the loads 142, without
-// A's stores 150.  With A's terms in shared memory as well, where the MMAs then
-// read twice as much, it takes 162.  CUDA-core tiles took 426 us for expert_up
-// alone and 758 for expert_down.
+// it) takes 149 us.  When it took 155, copies of the kernel without the MMAs took
+// 128, with half of them 133, without B's split and stores 142, without the loads
+// 142, without A's stores 150, and with A's terms in shared memory as well, where
+// the MMAs then read twice as much, 162.  CUDA-core tiles took 426 us for
+// expert_up alone and 758 for expert_down.
 //
 // One persistent CTA of 16 warps per SM (a 17th warp for the MMAs alone would
 // cut the registers per thread from 128 to 96).  Every warp loads A and B blocks

@@ -997,6 +997,9 @@ cudaError_t launch_gate(const GateArgs& a, bool bf16, cudaStream_t s, bool* rout
       p.pf_tile_rows = a.pf_tile_rows;
       p.pf_row_bytes = a.pf_row_bytes;
     }
+    // an upper bound (the CTAs of the decision kernel share SMs); the fused codec,
+    // its only reader, meets this gate at d = 1024 alone, where each of its widths
+    // fits beside it
     if (held_sms) *held_sms = (a.T + GD_BT_PLAIN - 1) / GD_BT_PLAIN;
     return bf16 ? launch_gate_partial<__nv_bfloat16>(a, p, O, s) : launch_gate_partial<float>(a, p, O, s);
   }
