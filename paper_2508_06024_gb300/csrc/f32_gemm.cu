@@ -54,6 +54,8 @@
 // in every row; with one sum after the other 274 and 2119).
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -621,13 +623,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
   }
 }
 
+// CTAs (split 1 of `sms` SMs) or clusters of `split` CTAs that run at once; 0
+// when such clusters cannot be placed.  Kept here per device beside max_clusters'
+// own table, whose search costs the host 0.1 us: a launch asks six times.
 template <int BN, int EPI>
-cudaError_t launch_bn(const GemmArgs& a, const FParams& p, long long tiles, cudaStream_t s) {
+int slots(int split, int sms) {
+  if (split == 1) return sms;
+  constexpr int DEVICES = 16;
+  static std::atomic<int> known[DEVICES][MAX_SPLIT + 1];  // one more than the answer; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev < DEVICES)
+    if (const int n = known[dev][split].load(std::memory_order_relaxed)) return n - 1;
+  const void* kernel = reinterpret_cast<const void*>(f32_gemm_kernel<BN, EPI>);
+  if (ensure_smem_attr(kernel, FCfg<BN>::SMEM) != cudaSuccess) return 0;
+  const int n = max_clusters(kernel, NUM_THREADS, FCfg<BN>::SMEM, split);
+  if (dev < DEVICES && n > 0) known[dev][split].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
+template <int BN, int EPI>
+cudaError_t launch_bn(const GemmArgs& a, const FParams& p, long long tiles, bool one_wave, cudaStream_t s) {
   using C = FCfg<BN>;
   auto* kernel = f32_gemm_kernel<BN, EPI>;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kernel), C::SMEM);
   if (e != cudaSuccess) return e;
-  const long long cap = sm_count() / p.split;
+  const int sms = sm_count();
+  const long long cap = one_wave ? sms / p.split : slots<BN, EPI>(p.split, sms);
   const int clusters = static_cast<int>(tiles < cap ? (tiles > 0 ? tiles : 1) : cap);
   KernelScope ks(a.name ? a.name : "gemm_f32", s);
   cudaLaunchConfig_t cfg{};
@@ -659,26 +681,40 @@ cudaError_t launch_bn(const GemmArgs& a, const FParams& p, long long tiles, cuda
 // (one per group of at most 0.8 x 128 rows, else half a partial tile per
 // group) times that decide.  So large calls take
 // 128-wide tiles, and calls with fewer tiles than SMs split K over a cluster.
+// A wave is what runs at once: 152 CTAs, 76 clusters of two, 36 of four (not 38:
+// a cluster's SMs lie in one GPC).  Taken as 38, 111 expected tiles were three
+// waves on paper and four on the GPU (layer with E = 8, d = 768, d_ff = 3072, T =
+// 994: 260 us against 221; T = 1057, 4 allowed 326 against 231; d = 512, d_ff =
+// 2048, T = 1585 239 against 175).  37 and 38 tiles still count as one wave: the
+// number is an expectation, and the next best choice is the slower one (d = 768,
+// T = 260: 143 us against 155; d = 512, d_ff = 2048, T = 400 129 against 134).
+// Such a launch has 38 clusters, of which those without a tile end at once.
 template <int EPI>
 cudaError_t launch_epi(const GemmArgs& a, FParams p, cudaStream_t s) {
   constexpr int DIV = EPI == EPI_SWIGLU ? 2 : 1;
   const int num_kb = (a.K + BK - 1) / BK;
+  const int sms = sm_count();
   const int ga = a.g_active > 0 ? a.g_active : a.G;
   const double rows = (double)a.max_rows / ga;  // expected rows per group
   const double m_tiles = a.G == 1 ? (double)((a.max_rows + BM - 1) / BM) : ga * (rows <= 0.8 * BM ? 1.0 : rows / BM + 0.5);
   double best = 0.0;
   int best_bn = 0;
+  bool best_one = false;
   for (int bn = 128; bn >= 64; bn /= 2) {
     const int nt = (a.N + bn / DIV - 1) / (bn / DIV);
     for (int sp = 1; sp <= MAX_SPLIT && sp <= num_kb; sp *= 2) {
       const int per = (num_kb + sp - 1) / sp;
       if ((num_kb + per - 1) / per != sp) continue;  // an empty K range
-      const double tiles = m_tiles * nt, slots = sm_count() / sp;
-      const double waves = static_cast<double>(static_cast<long long>(tiles / slots + 0.999));
+      const int at_once = bn == 128 ? slots<128, EPI>(sp, sms) : slots<64, EPI>(sp, sms);
+      if (at_once < 1) continue;
+      const double tiles = m_tiles * nt;
+      const bool one_wave = tiles <= 1.001 * (sms / sp);
+      const double waves = one_wave ? 1.0 : static_cast<double>(static_cast<long long>(tiles / at_once + 0.999));
       const double t = waves * (per * (bn == 128 ? 1.0 : 0.75) + 2.0 + (sp > 1 ? 1.0 : 0.0));
       if (!best_bn || t < best) {
         best = t;
         best_bn = bn;
+        best_one = one_wave;
         p.split = sp;
         p.kb_per_split = per;
         p.n_tiles_n = nt;
@@ -686,7 +722,7 @@ cudaError_t launch_epi(const GemmArgs& a, FParams p, cudaStream_t s) {
     }
   }
   const long long tiles = (a.max_rows / BM + a.G) * p.n_tiles_n;
-  return best_bn == 64 ? launch_bn<64, EPI>(a, p, tiles, s) : launch_bn<128, EPI>(a, p, tiles, s);
+  return best_bn == 64 ? launch_bn<64, EPI>(a, p, tiles, best_one, s) : launch_bn<128, EPI>(a, p, tiles, best_one, s);
 }
 
 }  // namespace

@@ -58,7 +58,7 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 }
 
 // Clusters of `cdim` CTAs of `kernel` that fit on the device at once (cached
-// per device and kernel); 0 when the query fails.
+// per device, kernel and size); 0 when the query fails.
 int max_clusters(const void* kernel, int threads, int smem, int cdim);
 
 // As launch_kernel, for `clusters` clusters of `cdim` CTAs.

@@ -925,21 +925,21 @@ int choose_bn(const GemmArgs& a, int epi, bool pair = false) {
 }  // namespace
 
 // Clusters of `cdim` CTAs of `kernel` that fit on the device at once (cached
-// per device and kernel); 0 when the query fails.
+// per device, kernel and size); 0 when the query fails.
 int max_clusters(const void* kernel, int threads, int smem, int cdim) {
   struct Entry {
     int dev;
     const void* kernel;
-    int n;
+    int cdim, n;
   };
   static std::mutex mu;
-  static Entry cache[32];
+  static Entry cache[64];
   static int used = 0;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < used; ++i)
-    if (cache[i].dev == dev && cache[i].kernel == kernel) return cache[i].n;
+    if (cache[i].dev == dev && cache[i].kernel == kernel && cache[i].cdim == cdim) return cache[i].n;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cdim * sm_count());
   cfg.blockDim = dim3(threads);
@@ -956,7 +956,7 @@ int max_clusters(const void* kernel, int threads, int smem, int cdim) {
     (void)cudaGetLastError();
     n = 0;
   }
-  if (used < 32) cache[used++] = Entry{dev, kernel, n};
+  if (used < 64) cache[used++] = Entry{dev, kernel, cdim, n};
   return n;
 }
 

@@ -51,6 +51,19 @@ def test_codec_f32_edges(T, d, r):
     _check(Xh, Z, Vd)
 
 
+# K = 512 split over clusters of four as long as their tiles make one wave (36 fit
+# at once, 38 are launched), of two beyond, and unsplit
+@pytest.mark.parametrize("tiles", [36, 37, 38, 39, 76, 77, 153])
+def test_f32_split_by_tile_count(tiles):
+    T, d, r = tiles * 128 - 5, 512, 64
+    X, Ve = _randn(1, T, d), _randn(2, r, d)
+    desc = C.make_desc(T=T, d=d, E=8, d_ff=8, k=1, dtype=C.F32, r=r)
+    Z = torch.full((T, r), float("nan"), device="cuda")
+    C.ec2moe_lr_encode(desc, X, Ve, Z)
+    assert C.ec2moe_last_device_error() == C.OK
+    _check(Z, X, Ve)
+
+
 def test_f32_rows_aligned_to_16_bytes_only():
     T, d, r = 150, 104, 72
     X = _randn(1, T * d + 4)[4:].view(T, d)  # 16-byte aligned, not 32
