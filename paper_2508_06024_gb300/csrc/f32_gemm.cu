@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f32_gemm_kernel(const FParams 
 
 // CTAs (split 1 of `sms` SMs) or clusters of `split` CTAs that run at once; 0
 // when such clusters cannot be placed.  Kept here per device beside max_clusters'
-// own table, whose search costs the host 0.1 us: a launch asks six times.
+// own table, as a launch asks up to five times.
 template <int BN, int EPI>
 int slots(int split, int sms) {
   if (split == 1) return sms;

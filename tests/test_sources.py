@@ -3,9 +3,10 @@
 No tensor or bulk copy goes to several CTAs at once: the library also runs with
 one rank per GPU (`bench.py` under torchrun), where such copies are not used.
 
-The read-only load path is for weights alone: with programmatic dependent launch
-a kernel starts while the one before still writes its activations, and PTX allows
-read-only loads only of memory that nobody writes while the kernel runs.
+Explicit read-only loads (ld.global.nc, __ldg) are for weights alone: with
+programmatic dependent launch a kernel starts while the one before still writes
+its activations, and PTX allows such loads only of memory that nobody writes while
+the kernel runs.
 """
 
 import pathlib
